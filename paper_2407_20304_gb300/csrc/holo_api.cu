@@ -79,6 +79,7 @@ constexpr int kErrWord = 8;
 struct holo_ctx {
   holo_geometry geo{};
   int n = 0, P = 0, J = 0, K = 0, chunk = 0;
+  int sms = 1;  // SMs of the context's device
   float ext = 1.f;
   double wref = 0.0;
   int functional = HOLO_F2_AMPLITUDE;
@@ -117,8 +118,9 @@ struct holo_ctx {
   holo::Tap* d_ytap = nullptr;
   holo::AdjTap* d_xadj = nullptr;
   holo::AdjTap* d_yadj = nullptr;
-  int2* d_lines = nullptr;      // line -> {plane, box row}
-  std::vector<int> rowstart;    // first line of each plane (host)
+  int2* d_lines = nullptr;      // line -> {plane, box row}, in (distance, angle, row) order
+  std::vector<int> rowstart;    // first line of plane (k, j) at [j * K + k] (host)
+  unsigned mid_x = 0;           // bit j: every box of distance j lies in the columns P/4 .. 3P/4
   int tap_stride = 0;
   size_t tap_bytes = 0;
   // data: the amplitudes of holo_set_data copied into pass B's column-blocked layout
@@ -250,7 +252,7 @@ void dfree(holo_ctx* c, void* p, size_t bytes) {
 bool is_pow2(int x) { return x > 0 && (x & (x - 1)) == 0; }
 
 // Pass B's Y stage: a TMA tensor map over ybuf viewed as a row-major [planes * maxbys][2n]
-// float matrix, boxes of 2C floats x kStageBox rows.  Used only where the driver provides
+// float matrix, boxes of 2C floats x stage_box(P) rows.  Used only where the driver provides
 // the encoder, n is even (16-byte row pitch) and the stage leaves pass B's resident blocks
 // per SM unchanged; otherwise pass B loads Y directly.
 using EncodeTiledFn = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*,
@@ -276,14 +278,15 @@ EncodeTiledFn encode_tiled() {
 holo_status encode_ystage(holo_ctx* c, int maxbys) {
   c->ystage = false;
   const int n = c->n, C = c->ops->pass_b_cols;
-  if (n % 2 || !c->ops->pass_b_stage_ok(n, maxbys)) return HOLO_OK;
+  if (n % 2 || !c->ops->pass_b_stage_ok(c->ops->half_form(n, c->probe_shift), maxbys))
+    return HOLO_OK;
   EncodeTiledFn enc = encode_tiled();
   if (!enc) return HOLO_OK;
   const long long rows = (long long)c->chunk * c->J * (c->ystride / n);
   CUtensorMap m;
   const cuuint64_t dims[2] = {(cuuint64_t)2 * n, (cuuint64_t)rows};
   const cuuint64_t strides[1] = {(cuuint64_t)n * sizeof(float2)};
-  const cuuint32_t box[2] = {(cuuint32_t)(2 * C), (cuuint32_t)holo::kStageBox};
+  const cuuint32_t box[2] = {(cuuint32_t)(2 * C), (cuuint32_t)holo::stage_box(c->P)};
   const cuuint32_t estr[2] = {1, 1};
   if (enc(&m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, c->ybuf, dims, strides, box, estr,
           CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
@@ -351,34 +354,37 @@ std::vector<float2> chirp_table(int P, double lambda, double dx, double z) {
   return c;
 }
 
-// Twiddle table in the layout of holo_fft.cuh for P = PB or 3 PB (PB a power of two):
-// radix-16 stage s with M(s) = PB/16^(s+1) > 1 contributes entries
-// [(k-1) M + mu] = exp(-2 pi i mu k 16^s / PB), k = 1..15; for P = 3 PB the radix-3 step
-// adds exp(-2 pi i r n / P) for r = 1, 2 (outer) and n < PB (inner).
+// Twiddle table of one line length (FP64).  P = 2^k, in the layout of holo_line.cuh (E values per
+// thread, T = P/E threads, second stage of T2 = min(T, E)): entries [l E + k1] =
+// exp(-2 pi i k1 2^l / (E T2)), l < log2 T2, k1 < E, then for T > E [t] = exp(-2 pi i t / P).
+// P = 3 PB, in the layout of holo_fft.cuh: radix-16 stage s with M(s) = PB/16^(s+1) > 1
+// contributes entries [(k-1) M + mu] = exp(-2 pi i mu k 16^s / PB), k = 1..15, then the radix-3
+// step adds exp(-2 pi i r n / P) for r = 1, 2 (outer) and n < PB (inner).
 std::vector<float2> twiddle_table(int P) {
   std::vector<float2> tw;
-  const int PB = P % 3 == 0 ? P / 3 : P;
+  const double pi = 3.14159265358979323846;
+  auto push = [&](double a) { tw.push_back(make_float2((float)std::cos(a), (float)std::sin(a))); };
+  if (P % 3) {
+    const int E = P >= 512 ? 32 : 16, T = P / E, T2 = std::min(T, E);
+    for (int m = 1; m < T2; m *= 2)
+      for (int k = 0; k < E; ++k) push(-2.0 * pi * (double)k * m / (E * T2));
+    if (T > E)
+      for (int t = 0; t < T; ++t) push(-2.0 * pi * (double)t / P);
+    return tw;
+  }
+  const int PB = P / 3;
   int log2p = 0;
   while ((1 << log2p) < PB) ++log2p;
-  const int n16 = log2p / 4;
-  const double pi = 3.14159265358979323846;
   long long L = 1;
-  for (int s = 0; s < n16; ++s) {
+  for (int s = 0; s < log2p / 4; ++s) {
     const long long M = PB / (L * 16);
     if (M > 1)
       for (int k = 1; k < 16; ++k)
-        for (long long mu = 0; mu < M; ++mu) {
-          const double a = -2.0 * pi * (double)(mu * k * L) / PB;
-          tw.push_back(make_float2((float)std::cos(a), (float)std::sin(a)));
-        }
+        for (long long mu = 0; mu < M; ++mu) push(-2.0 * pi * (double)(mu * k * L) / PB);
     L *= 16;
   }
-  if (PB != P)
-    for (int r = 1; r <= 2; ++r)
-      for (int nn = 0; nn < PB; ++nn) {
-        const double a = -2.0 * pi * (double)(r * nn) / P;
-        tw.push_back(make_float2((float)std::cos(a), (float)std::sin(a)));
-      }
+  for (int r = 1; r <= 2; ++r)
+    for (int nn = 0; nn < PB; ++nn) push(-2.0 * pi * (double)(r * nn) / P);
   return tw;
 }
 
@@ -550,8 +556,14 @@ PassArgs pass_args(holo_ctx* c, int k0, int nk, const void* psi) {
   a.yadj = c->d_yadj;
   a.tap_stride = c->tap_stride;
   a.lines = c->d_lines;
-  a.line0 = c->rowstart[(size_t)k0 * c->J];
-  a.nlines = c->rowstart[(size_t)(k0 + nk) * c->J] - a.line0;
+  const int G = c->ops->row_lines;
+  for (int j = 0; j < c->J; ++j) {
+    const size_t first = (size_t)j * c->K + k0;
+    a.seg_line0[j] = c->rowstart[first];
+    a.seg_cnt[j] = c->rowstart[first + nk] - c->rowstart[first];
+    a.seg_step[j + 1] = a.seg_step[j] + (a.seg_cnt[j] + G - 1) / G;
+  }
+  a.mid_x = c->mid_x;
   a.pass_b_items = c->ops->pass_b_groups(c->n);
   a.ymap = c->ystage && c->sched_stage != 0 ? c->d_ymap : nullptr;
   a.row_per_sm = c->sched_row_per_sm;
@@ -574,16 +586,18 @@ PassArgs pass_args(holo_ctx* c, int k0, int nk, const void* psi) {
 //                T = ext sum_kj r_kj (+ w_ref r_ref on the first part);
 //   eval_qgrad:  grad_q of the whole chunk from T and the per-plane conj(w) v.
 // Pass B's grid.  Whole column groups go to the blocks in rounds.  When that leaves a partial
-// last round, the (group, plane) items of that round can be spread over all blocks: by the
-// plane-split kernel (pb_split 1, no Y stage; the default when there are fewer than three full
-// rounds, i.e. small n) or by the staged kernel itself (pb_split 2).  The partial residual sums
-// of a split need tslots slots of [n][C] per block.
+// last round, the (group, plane) items of that round can be spread over all blocks (pb_split 1:
+// without the Y stage, 2: with it where it fits; automatic when there are fewer than three full
+// rounds, i.e. small n).  The partial residual sums of a split need tslots slots of [n][C] per
+// block.
 holo_status pass_b_grid(holo_ctx* c, PassArgs& a, bool gradient, int* nblocks) {
   const int groups = a.pass_b_items;
-  const int full = c->ops->pass_b_blocks(1 << 30, c->n, a.ymap ? a.max_box_rows : 0);
+  const int half = c->ops->half_form(c->n, c->probe_shift);
+  if (c->sched_split == 1) a.ymap = nullptr;
+  const int full = c->ops->pass_b_blocks(1 << 30, half, a.ymap ? a.max_box_rows : 0);
   const bool partial = groups % full != 0;
   if (c->sched_split < 0)
-    a.pb_split = partial && groups / full < 3 ? 1 : 0;
+    a.pb_split = partial && groups / full < 3 ? 2 : 0;
   else
     a.pb_split = partial ? c->sched_split : 0;
   a.tslots = 0;
@@ -592,8 +606,7 @@ holo_status pass_b_grid(holo_ctx* c, PassArgs& a, bool gradient, int* nblocks) {
     return HOLO_OK;
   }
   const long long per = (long long)a.J * a.nk;
-  const int nbx = a.pb_split == 2 ? full
-                                  : c->ops->pass_b_blocks_split((long long)groups * per, c->n);
+  const int nbx = (int)std::min((long long)full, std::max((long long)c->sms, groups * per / 2));
   const long long rounds = groups / nbx, tail = groups - rounds * nbx, titems = tail * per;
   const long long range = (titems + nbx - 1) / nbx;
   a.tslots = titems > 0 ? (int)((range + per - 1) / per + 1) : 0;
@@ -614,7 +627,7 @@ holo_status pass_b_grid(holo_ctx* c, PassArgs& a, bool gradient, int* nblocks) {
 
 holo_status eval_begin(holo_ctx* c, PassArgs& a) {
   PassTimer tm_red(c, HOLO_T_REDUCE);
-  const int nbx = c->ops->pass_b_blocks(a.pass_b_items, c->n, a.ymap ? a.max_box_rows : 0);
+  const int nbx = (int)c->part_cap - kRefBlocks;  // behind pass B's partials
   const long long n2 = (long long)c->n * c->n;
   if (a.k0 == 0 && c->wref != 0.0) {
     // reference residual first: pass B folds w_ref r_ref into the grad_q source
@@ -649,12 +662,10 @@ holo_status eval_planes(holo_ctx* c, PassArgs& a, bool gradient, bool first, int
     // T carries only the reference residual
     PassArgs ab = a;
     if (c->probe_shift) ab.ext = 0.f;
-    HOLO_LAUNCH(c, c->ops->pass_b(ab, gradient ? 1 : 0, nbx, c->stream));
-    // the last round's combine kernel of a split form (the staged split is compiled for the
-    // form without probe shifts only; with them pb_split 2 runs whole groups)
-    if (gradient && (a.pb_split == 1 || (a.pb_split == 2 && !c->probe_shift)) &&
-        a.pass_b_items % nbx)
-      c->launches++;
+    ab.adj = gradient ? 1 : 0;
+    HOLO_LAUNCH(c, c->ops->pass_b(ab, nbx, c->stream));
+    // (the combine kernel of a split last round)
+    if (gradient && a.pb_split && a.pass_b_items % nbx) c->launches++;
   }
   {
     PassTimer tm_red(c, HOLO_T_REDUCE);
@@ -708,8 +719,7 @@ holo_status eval_qsources(holo_ctx* c, const PassArgs& a, int acc) {
 
 // grad_q (= or +=) 2 [ D_{-zeta_0}(C* T) + sum_j D_{-omega_j}(G'_j) ] from the accumulators.
 // The row stage of every source runs into its own scratch rows; the column stage of all of
-// them is one k_cols_sum launch (one inverse transform per column for the sum).  Where the
-// sources' chirps do not fit its shared memory, each source runs its own column stage.
+// them is one k_cols_sum launch (one inverse transform per column for the sum).
 holo_status eval_qfinish(holo_ctx* c, float2* grad_q, int acc) {
   PassTimer tm_q(c, HOLO_T_QGRAD);
   const int P = c->P, n = c->n, lo = P / 2 - n / 2;
@@ -726,15 +736,6 @@ holo_status eval_qfinish(holo_ctx* c, float2* grad_q, int acc) {
     if (qb[1] <= 0 || qb[3] <= 0) continue;
     src[S++] = {c->d_gacc + c->gacc_off[j], qb[0], qb[1], qb[2], qb[3],
                 c->d_chirp_omega + (size_t)j * P};
-  }
-  if (S > c->ops->cols_sum_max()) {
-    for (int s = 0; s < S; ++s) {
-      holo_status st = dstep2d(c, src[s].in, src[s].r_lo, src[s].rows, src[s].c_lo, src[s].w,
-                               grad_q, 0, P, 0, P, src[s].chirp, 1, 2.f, s == 0 ? acc : 1);
-      if (st != HOLO_OK) return st;
-    }
-    c->q_pending = false;
-    return HOLO_OK;
   }
   size_t rows = 0;
   for (int s = 0; s < S; ++s) rows += (size_t)src[s].rows;
@@ -925,6 +926,15 @@ holo_status holo_create(const holo_geometry* geo, void* stream, holo_ctx** out) 
   c->wref = geo->w_ref;
   c->stream = (cudaStream_t)stream;
   c->ops = ops;
+  {
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&c->sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+        c->sms < 1) {
+      cudaGetLastError();
+      c->sms = 1;
+    }
+  }
   // Sec. 2 after Eq. fwd_model_cone3: m~_j = z_j/z_0, omega_j = (z_j - z_0)/m~_j,
   // zeta_j = z_j (Z - z_j)/Z; detector-side distance zhat_j = zeta_j / m~_j^2.
   const double z0 = geo->z[0];
@@ -1074,11 +1084,21 @@ holo_status build_planes(holo_ctx* c) {
     const double mt = c->mt[p % J];
     axis_taps(mt, teff[p * 2 + 1], n, P, d.bx0, d.bxs, &xt[p * stride], &xa[p * n]);
     axis_taps(mt, teff[p * 2 + 0], n, P, d.by0, d.bys, &yt[p * stride], &ya[p * n]);
-    c->rowstart[p + 1] = c->rowstart[p] + d.bys;
   }
-  std::vector<int2> lines((size_t)c->rowstart[np_all]);
-  for (size_t p = 0; p < np_all; ++p)
-    for (int r = 0; r < c->planes[p].bys; ++r) lines[(size_t)c->rowstart[p] + r] = make_int2((int)p, r);
+  std::vector<int2> lines;
+  c->mid_x = 0;
+  for (int j = 0; j < J; ++j) {
+    bool mid = true;
+    for (int k = 0; k < K; ++k) {
+      const size_t p = (size_t)k * J + j;
+      const PlaneDesc& d = c->planes[p];
+      c->rowstart[(size_t)j * K + k] = (int)lines.size();
+      for (int r = 0; r < d.bys; ++r) lines.push_back(make_int2((int)p, r));
+      mid = mid && d.bx0 >= P / 4 && d.bx0 + d.bxs <= 3 * P / 4;
+    }
+    if (mid) c->mid_x |= 1u << j;
+  }
+  c->rowstart[np_all] = (int)lines.size();
   holo_status st;
   {
     void* olds[] = {c->d_xtap, c->d_ytap, c->d_xadj, c->d_yadj, c->d_lines};
@@ -1113,7 +1133,9 @@ holo_status build_planes(holo_ctx* c) {
   const long long np = (long long)c->chunk * J;
   const size_t ybytes = sizeof(float2) * (size_t)(np * ystride);
   const size_t gbytes = sizeof(float2) * (size_t)(np * gkstride);
-  const long long parts = (long long)c->ops->pass_b_blocks(1 << 30, n, 0) + kRefBlocks + 1024;
+  const long long parts = (long long)std::max(c->ops->pass_b_blocks(1 << 30, 0, 0),
+                                              c->ops->pass_b_blocks(1 << 30, c->ops->half_form(n, 0), 0)) +
+                          kRefBlocks + 1024;
   if (ystride > c->ystride || gkstride > c->gkstride || !c->ybuf) {
     dfree(c, c->ybuf, sizeof(float2) * (size_t)(np * c->ystride));
     dfree(c, c->gkbuf, sizeof(float2) * (size_t)(np * c->gkstride));
@@ -1678,12 +1700,12 @@ holo_status holo_launch_count(const holo_ctx* c, long long* count) {
 // ------------------------------------------------------------------ batched evaluation
 
 // Work lists of one round of a batch: the r-th chunk of every problem that has one.  Problems
-// of one line length (and probe-shift form) share the launches of passes A, B and C; pass D
+// of one line length and form (n = P/2 or general) share the launches of passes A, B and C; pass D
 // has one launch for all.  Items are {index into the round's PassArgs, work index}.
 struct BatchGroup {
   const holo::Ops* ops = nullptr;
-  int shift = 0, max_n = 0, max_rows = 0, per_sm = 0;
-  std::vector<int2> rows, cols;  // pass A / C: {arg, first line}; pass B: {arg, block}
+  int half = 0, max_rows = 0, per_sm = 0;
+  std::vector<int2> rows, cols;  // pass A / C: {arg, block-step}; pass B: {arg, block}
   size_t off_rows = 0, off_cols = 0;
 };
 
@@ -1782,24 +1804,24 @@ holo_status holo_batch_prepare(holo_batch* b) {
       holo_status st = pass_b_grid(c, a, true, &nbx);
       if (st) return st;
       a.pb_blocks = nbx;
+      a.adj = 1;
       const int ai = (int)R.args.size();
       R.prob.push_back((int)i);
       R.args.push_back(a);
       R.nbx.push_back(nbx);
-      const int shift = a.ramp_x != nullptr;
+      const int half = c->ops->half_form(c->n, c->probe_shift);
       BatchGroup* g = nullptr;
       for (auto& x : R.groups)
-        if (x.ops == c->ops && x.shift == shift) g = &x;
+        if (x.ops == c->ops && x.half == half) g = &x;
       if (!g) {
         R.groups.emplace_back();
         g = &R.groups.back();
         g->ops = c->ops;
-        g->shift = shift;
+        g->half = half;
         g->per_sm = c->sched_row_per_sm;
       }
-      g->max_n = std::max(g->max_n, c->n);
       if (a.ymap) g->max_rows = std::max(g->max_rows, a.max_box_rows);
-      for (int base = 0; base < a.nlines; base += c->ops->row_lines) g->rows.push_back({ai, base});
+      for (int st = 0; st < a.seg_step[c->J]; ++st) g->rows.push_back({ai, st});
       for (int blk = 0; blk < nbx; ++blk) g->cols.push_back({ai, blk});
       for (int e = 0; e < nk * c->n; ++e) R.dits.push_back({ai, e});
     }
@@ -1871,11 +1893,10 @@ extern "C" holo_status holo_batch_gradient(holo_batch* b, void* stream) {
     }
     for (auto& g : R.groups)
       HOLO_CK(c0, g.ops->rows_multi(0, dargs, reinterpret_cast<const int2*>(dm + g.off_rows),
-                                    (int)g.rows.size(), g.shift, g.max_n, g.per_sm, s));
+                                    (int)g.rows.size(), g.half, g.per_sm, s));
     for (auto& g : R.groups)
       HOLO_CK(c0, g.ops->pass_b_multi(dargs, reinterpret_cast<const int2*>(dm + g.off_cols),
-                                      (int)g.cols.size(), na, 1, g.shift, g.max_n, g.max_rows, 0,
-                                      s));
+                                      (int)g.cols.size(), na, g.half, g.max_rows, 0, s));
     for (int ai = 0; ai < na; ++ai) {
       holo_ctx* c = b->ctx[R.prob[ai]];
       HOLO_LAUNCH(c, holo::launch_sum_f64(c->d_part, R.nbx[ai], c->d_red, 0, s));
@@ -1883,7 +1904,7 @@ extern "C" holo_status holo_batch_gradient(holo_batch* b, void* stream) {
     }
     for (auto& g : R.groups)
       HOLO_CK(c0, g.ops->rows_multi(1, dargs, reinterpret_cast<const int2*>(dm + g.off_rows),
-                                    (int)g.rows.size(), g.shift, g.max_n, g.per_sm, s));
+                                    (int)g.rows.size(), g.half, g.per_sm, s));
     HOLO_CK(c0, holo::launch_pass_d_multi(dargs, reinterpret_cast<const int2*>(dm + R.off_dits),
                                           (int)R.dits.size(), 16 * sms, s));
     // the probe gradient's sources are summed over the rounds and propagated once, in the

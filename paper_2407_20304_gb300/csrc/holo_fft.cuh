@@ -1,27 +1,24 @@
-// Register + shared-memory FFT engine for one line of length P: a power of two >= 16, or
-// three times one (P = 3 PB, PB >= 16).
+// Register + shared-memory FFT engine of the line lengths P = 3 PB (PB = 2^k, 16 .. 1024), and
+// the complex helpers shared with holo_line.cuh.
 //
 // The Fresnel operator D_z (Appendix A, Eq. defPz/defGz) is a circular convolution on
 // the P x P grid; with a separable chirp exp(-i pi lambda z (fx^2 + fy^2)) it factors into
 // one pass over rows and one over columns, each "FFT -> chirp -> inverse FFT" along a
-// line.  This header implements that line transform.
+// line.
 //
-// Layout.  A line is held by T = P/16 threads, 16 complex values per thread: thread t,
-// register c holds element t + T*c ("strided natural" layout).  The forward transform
-// is a mixed-radix decimation in frequency with radices 16, 16, ..., 16, r (r in
-// {2, 4, 8} when log2 P is not a multiple of 4); every stage is a DFT over one digit in
-// registers followed by a twiddle and a shared-memory exchange.  The thread/register
-// assignment of each stage is chosen so that the forward output is again in strided
-// natural order (register rho of thread t holds frequency t + T*rho), so a pointwise
-// multiplier in frequency needs no reordering and the inverse transform (the adjoint
-// stages in reverse order) consumes that layout directly and returns the same layout.
+// Sub-line of length PB: TB = PB/16 threads, 16 complex values per thread: thread t, register c
+// holds element t + TB c ("strided natural" layout).  The forward transform is a mixed-radix
+// decimation in frequency with radices 16, 16, ..., 16, r (r in {2, 4, 8} when log2 PB is not a
+// multiple of 4); every stage is a DFT over one digit in registers followed by a twiddle and a
+// shared-memory exchange.  The thread/register assignment of each stage is chosen so that the
+// forward output is again in strided natural order, so a pointwise multiplier in frequency needs
+// no reordering and the inverse transform (the adjoint stages in reverse order) consumes that
+// layout directly and returns the same layout.
 //
-// Exchanges write register k of thread t at t + T*k (contiguous per k) and read the
-// next stage's digit; addresses are padded a -> a + a/16 so both phases avoid shared
-// memory bank conflicts.  Twiddles come from a per-stage table in shared memory,
-// indexed [k-1][mu] so that consecutive threads read consecutive entries.
+// Exchanges write register k of thread t at t + TB k (contiguous per k) and read the next stage's
+// digit; addresses are padded a -> a + a/16 so both phases avoid shared memory bank conflicts.
 //
-// P = 3 PB.  The T = P/16 threads form three groups of TB = PB/16; thread t = q TB + i
+// P = 3 PB.  The T = P/16 threads form three groups of TB; thread t = q TB + i
 // holds element i + TB c + PB q (pos).  The forward transform first takes one radix-3
 // decimation-in-frequency step through shared memory: group q forms
 //   y_q[n] = W_P^{n q} (x[n] + W_3^q x[n + PB] + W_3^{2q} x[n + 2 PB]),  n = i + TB c,
@@ -31,11 +28,7 @@
 // adjoint steps in reverse order and returns the pos layout.
 //
 // Synchronisation: every thread of a line group calls the transform the same number of
-// times; the Sync policy is a block-wide barrier or a named barrier per line group.  The
-// buffer must be free when a transform starts.  It is free again when fft_inv returns; after
-// fft_fwd at P = 4096 other thread groups may still read their rows of the last (group-local)
-// exchange, so an fft_inv may follow directly (it starts on the same threads' rows) and any
-// other use of the buffer needs a barrier first.
+// times.  The buffer must be free when a transform starts and is free again when it returns.
 
 #pragma once
 
@@ -133,18 +126,12 @@ struct Fft {
   // radix-3 step: W_P^n and W_P^{2n}, n < PB, appended to both tables
   static constexpr int TW = TW_BASE + (R3 ? 2 * PB : 0);
   static constexpr int ROOTS = ROOTS_BASE + (R3 ? 2 * PB : 0);
-  // P = 4096: the exchange before the last radix-16 stage stays inside each group of 16
-  // threads t = 16a .. 16a + 15 (which every kernel keeps in one warp), so it needs a warp
-  // barrier only; the last stage then numbers its threads k1 + 16 a (see fwd_from).
-  static constexpr bool HW = !R3 && RB == 0 && N16 == 3;
-  static constexpr int HW_ROW = 17, HW_GROUP = 16 * 17;  // group region: 16 rows of 17
   // line element held in register c of thread t, and the frequency it holds after fft_fwd
   __host__ __device__ static constexpr int pos(int t, int c) {
     return R3 ? t % TB + TB * c + PB * (t / TB) : t + T * c;
   }
   __host__ __device__ static constexpr int fpos(int t, int c) {
-    return R3 ? 3 * (t % TB + TB * c) + t / TB
-              : (HW ? (t >> 4) + (T / 16) * (t & 15) + T * c : t + T * c);
+    return R3 ? 3 * (t % TB + TB * c) + t / TB : t + T * c;
   }
 };
 
@@ -248,72 +235,32 @@ __device__ __forceinline__ void dft_small(float2* u) {
 
 // --------------------------------------------------------------------- twiddle tables
 
-// Host-side layout of the shared twiddle table of one line length: for each radix-16
+// Host-side layout of the twiddle table of one line length P = 3 PB: for each radix-16
 // stage s with M(s) > 1, entries [(k-1) * M(s) + mu] = exp(-2 pi i mu k L(s) / PB),
-// k = 1..15, mu = 0..M(s)-1; for P = 3 PB then [n] = exp(-2 pi i n / P) and
+// k = 1..15, mu = 0..M(s)-1; then [n] = exp(-2 pi i n / P) and
 // [PB + n] = exp(-2 pi i 2n / P), n < PB.  Filled in FP64 on the host.
 
-template <int P>
-__device__ __forceinline__ void load_twiddles(float2* sm_tw, const float2* __restrict__ g_tw) {
-  for (int i = threadIdx.x; i < Fft<P>::TW; i += blockDim.x) sm_tw[i] = g_tw[i];
+// v[k] times the k-th power of r (its conjugate for INV), k = 1 .. 15: the powers by a product
+// tree of depth <= 4 (rounding error a few ulp).
+template <bool INV>
+__device__ __forceinline__ void pow_apply(float2 (&v)[16], float2 r) {
+  float2 w[16];
+  w[1] = r;
+  w[2] = cmul(r, r);
+  w[3] = cmul(w[2], r);
+  w[4] = cmul(w[2], w[2]);
+  w[5] = cmul(w[4], r);
+  w[6] = cmul(w[4], w[2]);
+  w[7] = cmul(w[4], w[3]);
+  w[8] = cmul(w[4], w[4]);
+#pragma unroll
+  for (int k = 9; k < 16; ++k) w[k] = cmul(w[8], w[k - 8]);
+#pragma unroll
+  for (int k = 1; k < 16; ++k) v[k] = INV ? cmulc(v[k], w[k]) : cmul(v[k], w[k]);
 }
 
-// --------------------------------------------------------------------- twiddle providers
-
-// TwTable: the per-stage table in shared memory, one load per twiddle.
-struct TwTable {
-  const float2* tw;
-  // radix-3 twiddle W_P^{(idx / PB + 1)(idx % PB)}
-  template <int P>
-  __device__ __forceinline__ float2 r3(int idx) const {
-    return tw[Fft<P>::TW_BASE + idx];
-  }
-  template <int P, int S>
-  __device__ __forceinline__ float2 get(int mu, int k) const {
-    return tw[Fft<P>::tw_off(S) + (k - 1) * Fft<P>::M(S) + mu];
-  }
-  template <int P, int S, bool INV>
-  __device__ __forceinline__ void apply(float2 (&v)[16], int mu) const {
-    const float2* w = tw + Fft<P>::tw_off(S) + mu;
-#pragma unroll
-    for (int k = 1; k < 16; ++k)
-      v[k] = INV ? cmulc(v[k], w[(k - 1) * Fft<P>::M(S)]) : cmul(v[k], w[(k - 1) * Fft<P>::M(S)]);
-  }
-};
-
-// TwPow: one root r = W_P^{mu L(S)} from the full table (entry k = 1), the powers r^k
-// by a product tree of depth <= 4 (rounding error a few ulp), no further loads.
-struct TwPow {
-  const float2* tw;
-  template <int P>
-  __device__ __forceinline__ float2 r3(int idx) const {
-    return tw[Fft<P>::TW_BASE + idx];
-  }
-  template <int P, int S, bool INV>
-  __device__ __forceinline__ void apply(float2 (&v)[16], int mu) const {
-    const float2 r = tw[Fft<P>::tw_off(S) + mu];
-    pow_apply<INV>(v, r);
-  }
-  template <bool INV>
-  __device__ __forceinline__ static void pow_apply(float2 (&v)[16], float2 r) {
-    float2 w[16];
-    w[1] = r;
-    w[2] = cmul(r, r);
-    w[3] = cmul(w[2], r);
-    w[4] = cmul(w[2], w[2]);
-    w[5] = cmul(w[4], r);
-    w[6] = cmul(w[4], w[2]);
-    w[7] = cmul(w[4], w[3]);
-    w[8] = cmul(w[4], w[4]);
-#pragma unroll
-    for (int k = 9; k < 16; ++k) w[k] = cmul(w[8], w[k - 8]);
-#pragma unroll
-    for (int k = 1; k < 16; ++k) v[k] = INV ? cmulc(v[k], w[k]) : cmul(v[k], w[k]);
-  }
-};
-
-// TwRoots: the same power tree from the compact root table (Fft<P>::ROOTS entries), which
-// is small enough to keep in shared memory next to the chirp.
+// TwRoots: the powers from the compact root table (Fft<P>::ROOTS entries: k = 1 of every
+// twiddled stage), which is small enough to keep in shared memory next to the chirp.
 struct TwRoots {
   const float2* roots;
   template <int P>
@@ -322,7 +269,7 @@ struct TwRoots {
   }
   template <int P, int S, bool INV>
   __device__ __forceinline__ void apply(float2 (&v)[16], int mu) const {
-    TwPow::pow_apply<INV>(v, roots[Fft<P>::roots_off(S) + mu]);
+    pow_apply<INV>(v, roots[Fft<P>::roots_off(S) + mu]);
   }
 };
 
@@ -343,34 +290,19 @@ __device__ __forceinline__ void load_roots(float2* sm_roots, const float2* __res
 
 // --------------------------------------------------------------------- stages
 
-// Barrier over the threads of one line group: the whole block, or a named barrier
-// (id >= 1) over the `count` threads of this line when several lines share a block.
+// Barrier over the threads of one line group: the whole block.
 struct SyncBlock {
   __device__ __forceinline__ void operator()() const { __syncthreads(); }
 };
-struct SyncNamed {
-  int id, count;
-  __device__ __forceinline__ void operator()() const {
-    asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(count) : "memory");
-  }
-};
-
 #define HOLO_SYNC() sync()
 
-template <int P, int S, class Sync = SyncBlock, class TW = TwTable>
+template <int P, int S, class Sync = SyncBlock, class TW = TwRoots>
 __device__ __forceinline__ void fwd_from(float2 (&v)[16], float2* __restrict__ sm, TW tw, int t,
                                          Sync sync = Sync()) {
   using F = Fft<P>;
   if constexpr (S < F::N16) {
     constexpr int M = F::M(S);
-    constexpr bool group_in = F::HW && S == F::N16 - 1, group_out = F::HW && S == F::N16 - 2;
-    if constexpr (group_in) {
-      // thread 16 a + k1 takes digit d0 of (a, k1) from the rows its group wrote; no barrier
-      // after the read: the only later writes to these rows come from the same threads
-      const float2* hr = sm + (t >> 4) * F::HW_GROUP + F::HW_ROW * (t & 15);
-#pragma unroll
-      for (int c = 0; c < 16; ++c) v[c] = hr[c];
-    } else if constexpr (S > 0) {
+    if constexpr (S > 0) {
       const int mu = t % M, ka = t / M;
 #pragma unroll
       for (int c = 0; c < 16; ++c) v[c] = sm[spad(c * M + mu + 16 * M * ka)];
@@ -378,13 +310,7 @@ __device__ __forceinline__ void fwd_from(float2 (&v)[16], float2* __restrict__ s
     }
     dft16<false>(v);
     if constexpr (M > 1) tw.template apply<P, S, false>(v, t % M);
-    if constexpr (group_out) {
-      // thread 16 a + mu holds digit k1 = k of (mu, a): row k, column mu of its group's region
-      float2* hr = sm + (t >> 4) * F::HW_GROUP + (t & 15);
-#pragma unroll
-      for (int k = 0; k < 16; ++k) hr[F::HW_ROW * k] = v[k];
-      __syncwarp();
-    } else if constexpr (S < F::NST - 1) {
+    if constexpr (S < F::NST - 1) {
 #pragma unroll
       for (int k = 0; k < 16; ++k) sm[spad(t + F::T * k)] = v[k];
       HOLO_SYNC();
@@ -406,7 +332,7 @@ __device__ __forceinline__ void fwd_from(float2 (&v)[16], float2* __restrict__ s
   }
 }
 
-template <int P, int S, class Sync = SyncBlock, class TW = TwTable>
+template <int P, int S, class Sync = SyncBlock, class TW = TwRoots>
 __device__ __forceinline__ void inv_from(float2 (&v)[16], float2* __restrict__ sm, TW tw, int t,
                                          Sync sync = Sync()) {
   using F = Fft<P>;
@@ -433,20 +359,8 @@ __device__ __forceinline__ void inv_from(float2 (&v)[16], float2* __restrict__ s
     constexpr int M = F::M(S);
     if constexpr (M > 1) tw.template apply<P, S, true>(v, t % M);
     dft16<true>(v);
-    if constexpr (F::HW && S == F::N16 - 1) {
-      // adjoint of the group exchange: thread 16 a + k1 writes its row, thread 16 a + mu
-      // reads column mu back
-      float2* hr = sm + (t >> 4) * F::HW_GROUP;
-#pragma unroll
-      for (int c = 0; c < 16; ++c) hr[F::HW_ROW * (t & 15) + c] = v[c];
-      __syncwarp();
-#pragma unroll
-      for (int k = 0; k < 16; ++k) v[k] = hr[F::HW_ROW * k + (t & 15)];
-      inv_from<P, S - 1, Sync, TW>(v, sm, tw, t, sync);
-    } else if constexpr (S > 0) {
+    if constexpr (S > 0) {
       const int mu = t % M, ka = t / M;
-      // other groups may still be reading their rows of the group exchange
-      if constexpr (F::HW && S == F::N16 - 2) HOLO_SYNC();
 #pragma unroll
       for (int c = 0; c < 16; ++c) sm[spad(c * M + mu + 16 * M * ka)] = v[c];
       HOLO_SYNC();
@@ -530,11 +444,6 @@ __device__ __forceinline__ void fft_fwd_with(float2 (&v)[16], float2* sm, TW tw,
   else
     fwd_from<P, 0, Sync, TW>(v, sm, tw, t, sync);
 }
-template <int P>
-__device__ __forceinline__ void fft_fwd(float2 (&v)[16], float2* sm, const float2* tw, int t) {
-  fft_fwd_with<P, SyncBlock, TwTable>(v, sm, TwTable{tw}, t, SyncBlock());
-}
-
 // Inverse DFT without the 1/P factor (the adjoint of fft_fwd): fpos in, pos out.
 template <int P, class Sync, class TW>
 __device__ __forceinline__ void fft_inv_with(float2 (&v)[16], float2* sm, TW tw, int t, Sync sync) {
@@ -543,9 +452,4 @@ __device__ __forceinline__ void fft_inv_with(float2 (&v)[16], float2* sm, TW tw,
   else
     inv_from<P, Fft<P>::N16, Sync, TW>(v, sm, tw, t, sync);
 }
-template <int P>
-__device__ __forceinline__ void fft_inv(float2 (&v)[16], float2* sm, const float2* tw, int t) {
-  fft_inv_with<P, SyncBlock, TwTable>(v, sm, TwTable{tw}, t, SyncBlock());
-}
-
 }  // namespace holo

@@ -12,7 +12,7 @@ namespace holo {
 // support of R0(psi - ext) on the P x P grid (rows [by0, by0+bys), cols [bx0, bx0+bxs)).
 // m~ is split into a high part with few significant bits (so m_hi * integer is exact in
 // FP32) and a low part; see axis_tap() in holo_kernels.cuh.
-struct PlaneDesc {
+struct alignas(16) PlaneDesc {
   float mt_hi, mt_lo;   // m~_j = mt_hi + mt_lo
   float ty, tx;         // sample shift t_kj (pixels), (y, x)
   int by0, bys;         // box rows
@@ -89,7 +89,7 @@ struct PassArgs {
   long long ystride;
   float2* tq;                  // [n][n]: ext sum_kj r_kj + w_ref r_ref (gradient only)
   int tq_accumulate;           // add to tq instead of overwriting (later parts of a chunk)
-  int pb_split;                // pass B: last round split by planes (k_pass_b_split)
+  int pb_split;                // pass B: last round of column groups split by planes
   float2* tpart;               // ... its partial S: per block tslots slots of [n][C]
   int tslots;
   int functional;              // 0: F2 (amplitudes, Eq. min1), 1: F1 (intensities, Eq. min2)
@@ -114,16 +114,20 @@ struct PassArgs {
   const AdjTap* xadj;          // [planes][n]: columns of psi
   const AdjTap* yadj;          // [planes][n]: rows of psi
   int tap_stride;
-  // rows of all planes in one flat list (plane p owns a contiguous run of its box rows):
-  // line -> {global plane, row within the plane's box}
+  // rows of all planes in one flat list in (distance, angle, box row) order:
+  // line -> {global plane, row within the plane's box}.  The chunk's lines of distance j are
+  // [seg_line0[j], seg_line0[j] + seg_cnt[j]); the row passes walk them in block-steps of
+  // row_lines lines, steps [seg_step[j], seg_step[j + 1]) of distance j.
   const int2* lines;           // [total box rows of all planes]
-  int line0, nlines;           // the chunk's lines: [line0, line0 + nlines)
+  int seg_line0[HOLO_MAX_DIST], seg_cnt[HOLO_MAX_DIST], seg_step[HOLO_MAX_DIST + 1];
+  unsigned mid_x;              // bit j: every box of distance j lies in the columns P/4 .. 3P/4
+  int adj;                     // pass B: 1 gradient (residual, adjoint), 0 forward only
   int pass_b_items;            // column groups of pass B
   int pb_blocks;               // pass-B grid of this problem (items of k_pass_b_multi)
   int row_per_sm;              // row passes: resident blocks per SM (0: as many as fit)
   // pass B stages each plane's Y tile [box rows][C columns] into shared memory by TMA
   // while the previous plane computes: tensor map over ybuf as a [planes * yrows][2n] float
-  // matrix (box 2C x kStageBox), or null for plain loads
+  // matrix (box 2C x stage_box(P)), or null for plain loads
   const void* ymap;
   int yrows;                   // rows per plane in ybuf (ystride / n)
   unsigned long long* err;     // device word, set when a bounded device wait gave up
@@ -134,8 +138,9 @@ struct PassArgs {
   const float2* ramp_y;
 };
 
-// Rows of one TMA box of pass B's Y stage (the tensor-map box limit is 256).
-constexpr int kStageBox = 256;
+// Rows of one TMA box of pass B's Y stage (at most 256): fewer copies for long lines, less rounding
+// of the stage's size for P = 1024.
+constexpr __host__ __device__ int stage_box(int P) { return P >= 2048 ? 256 : 128; }
 
 // Entry points implemented once per supported line length P.
 struct Ops {
@@ -143,28 +148,23 @@ struct Ops {
   cudaError_t (*rows)(const LineArgs&, const float2* tw, cudaStream_t);
   cudaError_t (*cols)(const LineArgs&, const float2* tw, cudaStream_t);
   cudaError_t (*pass_a)(const PassArgs&, cudaStream_t);
-  cudaError_t (*pass_b)(const PassArgs&, int with_adjoint, int nblocks, cudaStream_t);
+  cudaError_t (*pass_b)(const PassArgs&, int nblocks, cudaStream_t);
   cudaError_t (*pass_c)(const PassArgs&, cudaStream_t);
+  int (*half_form)(int n, int shift);       // 1: side n runs the passes' n = P/2 forms
   int (*pass_b_groups)(int n);              // column groups of pass B for side n
-  int (*pass_b_blocks)(int items, int n, int rows);  // persistent grid of pass B
-  int (*pass_b_blocks_split)(long long items, int n);  // ... of its plane-split form
-  int (*pass_b_stage_ok)(int n, int rows);  // 1: pass B may stage Y tiles of `rows` rows
+  int (*pass_b_blocks)(int items, int half, int rows);  // persistent grid of pass B
+  int (*pass_b_stage_ok)(int half, int rows);  // 1: pass B may stage Y tiles of `rows` rows
   int twiddle_count;
   int pass_b_cols;                          // columns per pass-B group (C)
-  int row_lines;                            // lines per block of the row passes (G)
+  int row_lines;                            // lines per block-step of the row passes (G)
   // several problems of this line length in one persistent launch (args, items in device
-  // memory; see k_pass_a_multi / k_pass_b_multi / k_pass_c_multi).  per_sm caps the resident
-  // blocks per SM (0: as many as fit); max_n / max_rows size the shared memory for the
-  // largest problem.
+  // memory; see k_rows_multi / k_pass_b_multi), all of them of one form (half).  per_sm caps the
+  // resident blocks per SM (0: as many as fit); max_rows sizes the Y stage.
   cudaError_t (*rows_multi)(int pass_c, const PassArgs* args, const int2* items, int nitems,
-                            int shift, int max_n, int per_sm, cudaStream_t);
+                            int half, int per_sm, cudaStream_t);
   cudaError_t (*pass_b_multi)(const PassArgs* args, const int2* items, int nitems, int nprob,
-                              int adj, int shift, int max_n, int max_rows, int per_sm,
-                              cudaStream_t);
-  // the summed column stage (k_cols_sum) and the most sources whose chirps fit its shared
-  // memory on the current device
-  cudaError_t (*cols_sum)(const SumArgs&, const float2* tw, cudaStream_t);
-  int (*cols_sum_max)();
+                              int half, int max_rows, int per_sm, cudaStream_t);
+  cudaError_t (*cols_sum)(const SumArgs&, const float2* tw, cudaStream_t);  // k_cols_sum
 };
 
 const Ops* ops_for(int P);

@@ -60,6 +60,15 @@ __device__ __forceinline__ void tma_load_2d(void* dst, const void* map, int x, i
       : "memory");
 }
 
+// 16-byte asynchronous copies of one thread into shared memory, and the wait for all of them.
+__device__ __forceinline__ void cp_async16(void* dst, const void* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"(smem_addr(dst)), "l"(src)
+               : "memory");
+}
+__device__ __forceinline__ void cp_async_wait() {
+  asm volatile("cp.async.wait_all;" ::: "memory");
+}
+
 // L2 prefetch (a hint: nothing is written to shared memory and nothing waits on it):
 // l2_prefetch_bulk fetches the 16-byte-aligned hull of [p, p + bytes) with one bulk request;
 // the hull must lie inside one allocation (every buffer here starts 256-byte aligned and
