@@ -192,7 +192,8 @@ struct holo_ctx {
 
 namespace {
 
-constexpr int kRefBlocks = 64;
+// (64 blocks took 160 us for the 2048^2 reference image, FP64 sums and all)
+constexpr int kRefBlocks = 512;
 
 holo_status fail(holo_ctx* c, holo_status s, const std::string& msg) {
   if (c) c->err = msg;
@@ -457,53 +458,35 @@ holo_status upload(holo_ctx* c, void* dst, const void* src, size_t bytes) {
   return HOLO_OK;
 }
 
-LineArgs line_args() {
-  LineArgs a;
-  std::memset(&a, 0, sizeof(a));
-  a.alpha = 1.f;
-  return a;
+// Source i of a line launch: `nlines` lines of positions [in_lo, in_lo + in_len), written at
+// [out_lo, out_lo + out_len).  rows: element (line, pos) at line * pitch + pos; columns: at pos *
+// pitch + line.
+void add_source(LineArgs& a, bool rows, const float2* in, long long in_pitch, int in_lo, int in_len,
+                float2* out, long long out_pitch, int out_lo, int out_len, int nlines,
+                const float2* chirp, int conj) {
+  holo::LineSource& s = a.src[a.S++];
+  s.in = in;
+  s.in_line_stride = rows ? in_pitch : 1;
+  s.in_step = rows ? 1 : in_pitch;
+  s.in_lo = in_lo;
+  s.in_len = in_len;
+  s.out = out;
+  s.out_line_stride = rows ? out_pitch : 1;
+  s.out_step = rows ? 1 : out_pitch;
+  s.out_lo = out_lo;
+  s.out_len = out_len;
+  s.nlines = nlines;
+  s.chirp = chirp;
+  s.conj_chirp = conj;
 }
 
-// 2D D_z of a field given as `rows` rows of width `w` occupying P-grid rows
-// [r_lo, r_lo + rows) and columns [c_lo, c_lo + w); the result keeps P-grid rows
-// [or_lo, or_lo + orows) and columns [oc_lo, oc_lo + ocols), written densely with row
-// pitch ocols, as out = alpha D(in) (+ out when accumulate).  Rows first, then columns.
-holo_status dstep2d(holo_ctx* c, const float2* in, int r_lo, int rows, int c_lo, int w,
-                    float2* out, int or_lo, int orows, int oc_lo, int ocols, const float2* chirp,
-                    int conj, float alpha, int accumulate) {
+// D_z of a P x P field (in == out allowed): rows into the scratch plane, then columns.
+holo_status dstep2d(holo_ctx* c, const float2* in, float2* out, const float2* chirp, int conj) {
   const int P = c->P;
-  LineArgs a = line_args();
-  a.in = in;
-  a.in_line_stride = w;
-  a.in_step = 1;
-  a.in_lo = c_lo;
-  a.in_len = w;
-  a.out = c->d_scratch;  // [rows][ocols]
-  a.out_line_stride = ocols;
-  a.out_step = 1;
-  a.out_lo = oc_lo;
-  a.out_len = ocols;
-  a.nlines = rows;
-  a.chirp = chirp;
-  a.conj_chirp = conj;
+  LineArgs a{}, b{};
+  add_source(a, true, in, P, 0, P, c->d_scratch, P, 0, P, P, chirp, conj);
   HOLO_LAUNCH(c, c->ops->rows(a, c->d_tw, c->stream));
-  LineArgs b = line_args();
-  b.in = c->d_scratch;
-  b.in_line_stride = 1;
-  b.in_step = ocols;
-  b.in_lo = r_lo;
-  b.in_len = rows;
-  b.out = out;
-  b.out_line_stride = 1;
-  b.out_step = ocols;
-  b.out_lo = or_lo;
-  b.out_len = orows;
-  b.nlines = ocols;
-  b.chirp = chirp;
-  b.conj_chirp = conj;
-  b.alpha = alpha;
-  b.accumulate = accumulate;
-  (void)P;
+  add_source(b, false, c->d_scratch, P, 0, P, out, P, 0, P, P, chirp, conj);
   HOLO_LAUNCH(c, c->ops->cols(b, c->d_tw, c->stream));
   return HOLO_OK;
 }
@@ -626,21 +609,24 @@ holo_status pass_b_grid(holo_ctx* c, PassArgs& a, bool gradient, int* nblocks) {
 }
 
 holo_status eval_begin(holo_ctx* c, PassArgs& a) {
+  if (a.k0 != 0 || c->wref == 0.0) return HOLO_OK;
   PassTimer tm_red(c, HOLO_T_REDUCE);
-  const int nbx = (int)c->part_cap - kRefBlocks;  // behind pass B's partials
-  const long long n2 = (long long)c->n * c->n;
-  if (a.k0 == 0 && c->wref != 0.0) {
-    // reference residual first: pass B folds w_ref r_ref into the grad_q source
-    HOLO_LAUNCH(c, holo::launch_ref_residual(c->d_b, c->sqrt_dref, n2, c->d_rref,
-                                             c->d_part + nbx, kRefBlocks, c->functional,
-                                             c->stream));
-    HOLO_LAUNCH(c, holo::launch_sum_f64(c->d_part + nbx, kRefBlocks, c->d_red + 1, 0, c->stream));
-    a.rref = c->d_rref;
-  } else {
-    // no reference term in this call: red[1] = 0 (a sum over nothing, by a kernel rather than a
-    // memset, which could wait behind a host-buffer call's copies)
-    HOLO_LAUNCH(c, holo::launch_sum_f64(c->d_part, 0, c->d_red + 1, 0, c->stream));
-  }
+  // reference residual first: pass B folds w_ref r_ref into the grad_q source; its loss partials
+  // lie behind pass B's
+  HOLO_LAUNCH(c, holo::launch_ref_residual(c->d_b, c->sqrt_dref, (long long)c->n * c->n, c->d_rref,
+                                           c->d_part + c->part_cap - kRefBlocks, kRefBlocks,
+                                           c->functional, c->stream));
+  a.rref = c->d_rref;
+  return HOLO_OK;
+}
+
+// The loss of one part of an evaluation from pass B's nbx partials (and, on the first part of a
+// call whose chunk has k0 == 0, the reference partials).
+holo_status eval_loss(holo_ctx* c, const PassArgs& a, int nbx, bool first, int acc) {
+  const bool ref = first && a.rref != nullptr;
+  HOLO_LAUNCH(c, holo::launch_loss(c->d_part, nbx, c->d_part + c->part_cap - kRefBlocks,
+                                   ref ? kRefBlocks : 0, c->d_red, c->wref, acc, first ? 1 : 0,
+                                   c->stream));
   return HOLO_OK;
 }
 
@@ -669,9 +655,8 @@ holo_status eval_planes(holo_ctx* c, PassArgs& a, bool gradient, bool first, int
   }
   {
     PassTimer tm_red(c, HOLO_T_REDUCE);
-    HOLO_LAUNCH(c, holo::launch_sum_f64(c->d_part, nbx, c->d_red, 0, c->stream));
-    HOLO_LAUNCH(c, holo::launch_loss_total(c->d_red, first ? c->wref : 0.0, acc, first ? 1 : 0,
-                                           c->stream));
+    holo_status st = eval_loss(c, a, nbx, first, acc);
+    if (st) return st;
   }
   if (!gradient) return HOLO_OK;
   {
@@ -706,20 +691,21 @@ holo_status eval_qsources(holo_ctx* c, const PassArgs& a, int acc) {
     c->gacc_bytes = need;
     acc = 0;
   }
+  holo::ReduceArgs r{};
+  r.accumulate = acc;
   for (int j = 0; j < c->J; ++j) {
     c->gacc_off[j] = off[j] / sizeof(float2);
-    const int* qb = c->qbox[j];
-    if (qb[1] <= 0 || qb[3] <= 0) continue;
-    HOLO_LAUNCH(c, holo::launch_reduce_g(a, c->d_gacc + c->gacc_off[j], j, qb[0], qb[1], qb[2],
-                                         qb[3], qb[3], qb[0], qb[2], acc, c->stream));
+    r.out[j] = c->d_gacc + c->gacc_off[j];
+    for (int i = 0; i < 4; ++i) r.box[j][i] = c->qbox[j][i];
   }
+  HOLO_LAUNCH(c, holo::launch_reduce_g(a, r, c->stream));
   c->q_pending = true;
   return HOLO_OK;
 }
 
 // grad_q (= or +=) 2 [ D_{-zeta_0}(C* T) + sum_j D_{-omega_j}(G'_j) ] from the accumulators.
-// The row stage of every source runs into its own scratch rows; the column stage of all of
-// them is one k_cols_sum launch (one inverse transform per column for the sum).
+// The row stage of every source runs into its own scratch rows (one launch); the column stage of
+// all of them is one k_cols_sum launch (one inverse transform per column for the sum).
 holo_status eval_qfinish(holo_ctx* c, float2* grad_q, int acc) {
   PassTimer tm_q(c, HOLO_T_QGRAD);
   const int P = c->P, n = c->n, lo = P / 2 - n / 2;
@@ -750,29 +736,18 @@ holo_status eval_qfinish(holo_ctx* c, float2* grad_q, int acc) {
   }
   holo::SumArgs sa;
   std::memset(&sa, 0, sizeof(sa));
+  LineArgs la{};
   size_t off = 0;
   for (int s = 0; s < S; ++s) {
-    LineArgs a = line_args();
-    a.in = src[s].in;
-    a.in_line_stride = src[s].w;
-    a.in_step = 1;
-    a.in_lo = src[s].c_lo;
-    a.in_len = src[s].w;
-    a.out = c->d_qscr + off;  // [rows][P]
-    a.out_line_stride = P;
-    a.out_step = 1;
-    a.out_lo = 0;
-    a.out_len = P;
-    a.nlines = src[s].rows;
-    a.chirp = src[s].chirp;
-    a.conj_chirp = 1;
-    HOLO_LAUNCH(c, c->ops->rows(a, c->d_tw, c->stream));
+    add_source(la, true, src[s].in, src[s].w, src[s].c_lo, src[s].w, c->d_qscr + off, P, 0, P,
+               src[s].rows, src[s].chirp, 1);
     sa.in[s] = c->d_qscr + off;
     sa.r_lo[s] = src[s].r_lo;
     sa.rows[s] = src[s].rows;
     sa.chirp[s] = src[s].chirp;
     off += (size_t)src[s].rows * P;
   }
+  HOLO_LAUNCH(c, c->ops->rows(la, c->d_tw, c->stream));
   sa.S = S;
   sa.conj_chirp = 1;
   sa.alpha = 2.f;
@@ -1262,23 +1237,25 @@ holo_status holo_set_data(holo_ctx* c, const float* sqrt_d, const float* sqrt_dr
 holo_status holo_set_probe(holo_ctx* c, const void* q) {
   if (!c || !q) return fail(c, HOLO_ERR_ARG, "null probe");
   const int P = c->P, n = c->n, lo = P / 2 - n / 2;
-  const size_t plane = sizeof(float2) * (size_t)P * P;
   PassTimer tm(c, HOLO_T_PROBE);
   // p_0 = q (omega_0 = 0), copied by a kernel: a copy engine may still be busy with the
   // host->device copies of a host-buffer call
-  (void)plane;
   HOLO_LAUNCH(c, holo::launch_scale_add(c->d_pj, (const float2*)q, 1.f, (long long)P * P, 0,
                                         c->stream));
-  holo_status st;
+  // p_j = D_{omega_j}(q) (Eq. fwd_model_cone3) and b = C D_{zeta_0}(q), the probe on the detector
+  // without the sample (Sec. 2): the rows of every distance in one launch (p_j's into p_j itself,
+  // b's detector columns into the scratch plane), then their columns in another
+  LineArgs a{}, b{};
   for (int j = 1; j < c->J; ++j) {
-    // p_j = D_{omega_j}(q)  (Eq. fwd_model_cone3)
-    st = dstep2d(c, (const float2*)q, 0, P, 0, P, c->d_pj + (size_t)j * P * P, 0, P, 0, P,
-                 c->d_chirp_omega + (size_t)j * P, 0, 1.f, 0);
-    if (st != HOLO_OK) return st;
+    float2* pj = c->d_pj + (size_t)j * P * P;
+    const float2* ch = c->d_chirp_omega + (size_t)j * P;
+    add_source(a, true, (const float2*)q, P, 0, P, pj, P, 0, P, P, ch, 0);
+    add_source(b, false, pj, P, 0, P, pj, P, 0, P, P, ch, 0);
   }
-  // b = C D_{zeta_0}(q): the probe on the detector without the sample (Sec. 2)
-  st = dstep2d(c, (const float2*)q, 0, P, 0, P, c->d_b, lo, n, lo, n, c->d_chirp_zeta0, 0, 1.f, 0);
-  if (st != HOLO_OK) return st;
+  add_source(a, true, (const float2*)q, P, 0, P, c->d_scratch, n, lo, n, P, c->d_chirp_zeta0, 0);
+  add_source(b, false, c->d_scratch, n, 0, P, c->d_b, n, lo, n, n, c->d_chirp_zeta0, 0);
+  HOLO_LAUNCH(c, c->ops->rows(a, c->d_tw, c->stream));
+  HOLO_LAUNCH(c, c->ops->cols(b, c->d_tw, c->stream));
   c->have_probe = true;
   return HOLO_OK;
 }
@@ -1501,12 +1478,11 @@ holo_status holo_finish_q(holo_ctx* c, void* grad_q, unsigned flags) {
 
 holo_status holo_propagate(holo_ctx* c, const void* in, void* out, double z) {
   if (!c || !in || !out || !std::isfinite(z)) return fail(c, HOLO_ERR_ARG, "bad argument");
-  const int P = c->P;
-  auto ch = chirp_table(P, c->geo.wavelength, c->geo.pixel, z);
-  holo_status st = upload(c, c->d_chirp_tmp, ch.data(), sizeof(float2) * P);
-  if (st) return st;
-  return dstep2d(c, (const float2*)in, 0, P, 0, P, (float2*)out, 0, P, 0, P, c->d_chirp_tmp, 0,
-                 1.f, 0);
+  // the chirp is made on the device: at P = 4096 the host's table, its copy and the wait for it
+  // took 100 of 265 us
+  HOLO_LAUNCH(c, holo::launch_chirp(c->d_chirp_tmp, c->P, c->geo.wavelength, c->geo.pixel, z,
+                                    c->stream));
+  return dstep2d(c, (const float2*)in, (float2*)out, c->d_chirp_tmp, 0);
 }
 
 holo_status holo_dot(holo_ctx* c, const void* a, const void* b, long long n, double* re_out) {
@@ -1633,10 +1609,8 @@ holo_status holo_upsample2(const void* in, long long count, int n, void* out, vo
 
 holo_status holo_initial_probe(holo_ctx* c, const float* sqrt_dref, void* q_out) {
   if (!c || !sqrt_dref || !q_out) return fail(c, HOLO_ERR_ARG, "null argument");
-  const int P = c->P;
-  HOLO_LAUNCH(c, holo::launch_embed_edge(sqrt_dref, c->n, P, (float2*)q_out, c->stream));
-  return dstep2d(c, (const float2*)q_out, 0, P, 0, P, (float2*)q_out, 0, P, 0, P,
-                 c->d_chirp_zeta0, 1, 1.f, 0);
+  HOLO_LAUNCH(c, holo::launch_embed_edge(sqrt_dref, c->n, c->P, (float2*)q_out, c->stream));
+  return dstep2d(c, (const float2*)q_out, (float2*)q_out, c->d_chirp_zeta0, 1);
 }
 
 holo_status holo_set_functional(holo_ctx* c, int functional) {
@@ -1899,8 +1873,7 @@ extern "C" holo_status holo_batch_gradient(holo_batch* b, void* stream) {
                                       (int)g.cols.size(), na, g.half, g.max_rows, 0, s));
     for (int ai = 0; ai < na; ++ai) {
       holo_ctx* c = b->ctx[R.prob[ai]];
-      HOLO_LAUNCH(c, holo::launch_sum_f64(c->d_part, R.nbx[ai], c->d_red, 0, s));
-      HOLO_LAUNCH(c, holo::launch_loss_total(c->d_red, c->wref, acc, 1, s));
+      if ((st = eval_loss(c, R.args[ai], R.nbx[ai], true, acc))) return st;
     }
     for (auto& g : R.groups)
       HOLO_CK(c0, g.ops->rows_multi(1, dargs, reinterpret_cast<const int2*>(dm + g.off_rows),

@@ -134,9 +134,11 @@ __global__ void __launch_bounds__(256) k_pass_d_multi(const PassArgs* __restrict
 // together (the additions stay in angle order).
 constexpr int kReduceEpt = 4;
 constexpr int kReduceTile = 128;
-__global__ void __launch_bounds__(256) k_reduce_g(PassArgs a, float2* Gp, int j, int row0, int nrows,
-                                                  int col0, int ncols, int opitch, int orow0,
-                                                  int ocol0, int accumulate) {
+__global__ void __launch_bounds__(256) k_reduce_g(const __grid_constant__ PassArgs a,
+                                                  const __grid_constant__ ReduceArgs r) {
+  const int j = blockIdx.y;
+  const int row0 = r.box[j][0], nrows = r.box[j][1], col0 = r.box[j][2], ncols = r.box[j][3];
+  if ((long long)blockIdx.x * blockDim.x * kReduceEpt >= (long long)nrows * ncols) return;
   __shared__ int4 box[kReduceTile];
   const long long total = (long long)nrows * ncols;
   const long long base = (long long)blockIdx.x * blockDim.x * kReduceEpt + threadIdx.x;
@@ -173,8 +175,8 @@ __global__ void __launch_bounds__(256) k_reduce_g(PassArgs a, float2* Gp, int j,
   for (int e = 0; e < kReduceEpt; ++e) {
     const long long idx = base + (long long)e * blockDim.x;
     if (idx < total) {
-      float2* o = Gp + (long long)(Y[e] - orow0) * opitch + (X[e] - ocol0);
-      *o = accumulate ? cadd(*o, acc[e]) : acc[e];
+      float2* o = r.out[j] + idx;
+      *o = r.accumulate ? cadd(*o, acc[e]) : acc[e];
     }
   }
 }
@@ -306,15 +308,40 @@ __global__ void k_sum_f64(const double* __restrict__ part, int count, double* ou
   if (threadIdx.x == 0) *out = accumulate ? *out + s : s;
 }
 
-// Running loss of the context: red[3] = (acc ? red[3] : 0) + red[0] + wref red[1].
-// red[0]: plane loss of the last launch group, red[1]: reference term.  red[3] is the
-// running total across calls (holo_read_loss), red[7] the total of the current call.
-__global__ void k_loss_total(double* red, double wref, int acc, int first) {
-  if (threadIdx.x == 0 && blockIdx.x == 0) {
-    const double l = red[0] + wref * red[1];
+// Loss of one part of an evaluation (single block): red[0] = sum of the plane partials; on the
+// first part red[1] = sum of the reference partials (0 without any); then the running total across
+// calls (holo_read_loss) red[3] = (acc ? red[3] : 0) + red[0] + wref red[1] and the current call's
+// red[7].  (One launch where two sums and a total took three: 25 us of the tiny gradient.)
+__global__ void k_loss(const double* __restrict__ part, int count,
+                       const double* __restrict__ refpart, int refcount, double* red, double wref,
+                       int acc, int first) {
+  __shared__ double sh[32];
+  double x = 0.0, y = 0.0;
+  for (int i = threadIdx.x; i < count; i += blockDim.x) x += part[i];
+  if (first)
+    for (int i = threadIdx.x; i < refcount; i += blockDim.x) y += refpart[i];
+  const double s0 = block_sum_f64(x, sh);
+  __syncthreads();
+  const double s1 = block_sum_f64(y, sh);
+  if (threadIdx.x == 0) {
+    red[0] = s0;
+    if (first) red[1] = s1;
+    const double l = s0 + (first ? wref * s1 : 0.0);
     red[3] = (acc ? red[3] : 0.0) + l;
     red[7] = (first ? 0.0 : red[7]) + l;
   }
+}
+
+// The chirp table of one distance (FP64; entry k at frequency k/(P dx), k in [-P/2, P/2)).
+__global__ void k_chirp(float2* __restrict__ out, int P, double lambda, double dx, double z) {
+  const int k = blockIdx.x * blockDim.x + threadIdx.x;
+  if (k >= P) return;
+  const double kk = k < P / 2 ? k : k - P;
+  const double f = kk / (P * dx);
+  const double ph = -3.14159265358979323846 * lambda * z * f * f;
+  double sn, cs;
+  sincos(ph, &sn, &cs);
+  out[k] = make_float2((float)(cs / P), (float)(sn / P));
 }
 
 // Re <a, b> = Re sum conj(a) b: FP32 products summed in FP32 over at most 16 elements per
@@ -434,12 +461,6 @@ __global__ void k_scale_add(float2* __restrict__ out, const float2* __restrict__
   }
 }
 
-__global__ void k_fill_zero(float2* __restrict__ out, long long n) {
-  for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n;
-       e += (long long)gridDim.x * blockDim.x)
-    out[e] = make_float2(0.f, 0.f);
-}
-
 int grid_for(long long n) {
   long long b = (n + kThreads - 1) / kThreads;
   if (b > 152 * 16) b = 152 * 16;
@@ -461,15 +482,15 @@ cudaError_t launch_pass_d_multi(const PassArgs* args, const int2* items, int nit
   return cudaGetLastError();
 }
 
-cudaError_t launch_reduce_g(const PassArgs& a, float2* out, int j, int row0, int nrows, int col0,
-                            int ncols, int opitch, int orow0, int ocol0, int accumulate,
-                            cudaStream_t s) {
-  const long long total = (long long)nrows * ncols;
-  if (total <= 0) return cudaSuccess;
+cudaError_t launch_reduce_g(const PassArgs& a, const ReduceArgs& r, cudaStream_t s) {
+  long long most = 0;
+  for (int j = 0; j < a.J; ++j) {
+    const long long total = (long long)r.box[j][1] * r.box[j][3];
+    most = most > total ? most : total;
+  }
+  if (most <= 0) return cudaSuccess;
   const long long per = 256LL * kReduceEpt;
-  k_reduce_g<<<(unsigned)((total + per - 1) / per), 256, 0, s>>>(a, out, j, row0, nrows, col0,
-                                                                 ncols, opitch, orow0, ocol0,
-                                                                 accumulate);
+  k_reduce_g<<<dim3((unsigned)((most + per - 1) / per), (unsigned)a.J), 256, 0, s>>>(a, r);
   return cudaGetLastError();
 }
 
@@ -527,8 +548,14 @@ cudaError_t launch_sum_f64(const double* part, int count, double* out, int accum
   return cudaGetLastError();
 }
 
-cudaError_t launch_loss_total(double* red, double wref, int acc, int first, cudaStream_t s) {
-  k_loss_total<<<1, 32, 0, s>>>(red, wref, acc, first);
+cudaError_t launch_loss(const double* part, int count, const double* refpart, int refcount,
+                        double* red, double wref, int acc, int first, cudaStream_t s) {
+  k_loss<<<1, 1024, 0, s>>>(part, count, refpart, refcount, red, wref, acc, first);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_chirp(float2* out, int P, double lambda, double dx, double z, cudaStream_t s) {
+  k_chirp<<<(P + 63) / 64, 64, 0, s>>>(out, P, lambda, dx, z);
   return cudaGetLastError();
 }
 
@@ -576,12 +603,6 @@ cudaError_t launch_scale_add(float2* out, const float2* in, float alpha, long lo
                              int accumulate, cudaStream_t s) {
   if (n <= 0) return cudaSuccess;
   k_scale_add<<<grid_for(n), kThreads, 0, s>>>(out, in, alpha, n, accumulate);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_fill_zero(float2* out, long long n, cudaStream_t s) {
-  if (n <= 0) return cudaSuccess;
-  k_fill_zero<<<grid_for(n), kThreads, 0, s>>>(out, n);
   return cudaGetLastError();
 }
 

@@ -35,28 +35,32 @@ struct AdjTap {
   int pad;
 };
 
-// Generic line D-step over rows or columns of a strided complex array.
-// The line's nonzero input occupies P-grid positions [in_lo, in_lo + in_len) and is
-// read from in[line_in_base + (pos - in_lo) * in_step]; outside, the input is zero.
-// The output is written for positions [out_lo, out_lo + out_len) to
-// out[line_out_base + (pos - out_lo) * out_step], as out = alpha * D + beta * out.
-struct LineArgs {
+// Line D-steps over the rows or columns of several sources in one launch.  A source's line i reads
+// P-grid positions [in_lo, in_lo + in_len) from in[i in_line_stride + (pos - in_lo) in_step] (zero
+// elsewhere) and writes positions [out_lo, out_lo + out_len) to out[i out_line_stride + (pos -
+// out_lo) out_step].  in and out of one source may be the same array where each thread's elements
+// are (same strides and ranges).
+constexpr int kMaxSumSources = 1 + HOLO_MAX_DIST;
+struct LineSource {
   const float2* in;
   float2* out;
   long long in_line_stride, in_step;     // element offsets
   long long out_line_stride, out_step;
   int nlines;
   int in_lo, in_len, out_lo, out_len;
-  const float2* chirp;                   // P entries, exp(-i pi lambda z f^2) / P
   int conj_chirp;                        // 1: multiply by conj(chirp) (distance -z)
-  float alpha;
-  int accumulate;                        // 1: out += alpha * D(...)
+  const float2* chirp;                   // P entries, exp(-i pi lambda z f^2) / P
+};
+struct LineArgs {
+  int S;                                 // sources, 1 .. kMaxSumSources
+  int step[kMaxSumSources + 1];          // block-steps of source s: [step[s], step[s + 1]) (set
+                                         // by the launcher)
+  LineSource src[kMaxSumSources];
 };
 
 // The column stage of sum_s D_s(x_s) over several sources whose row stage already ran: per
 // column of the P x P grid, the transforms of the sources' columns times their chirps are
 // summed and transformed back once (see k_cols_sum).
-constexpr int kMaxSumSources = 1 + HOLO_MAX_DIST;
 struct SumArgs {
   int S;                                     // sources, 1 .. kMaxSumSources
   const float2* in[kMaxSumSources];          // source s: rows [r_lo, r_lo + rows) of the grid,
@@ -178,11 +182,14 @@ cudaError_t launch_direction_step_dot(float2* x, float2* eta, const float2* g, f
                                       cudaStream_t s);
 cudaError_t launch_pass_d_multi(const PassArgs* args, const int2* items, int nitems, int nblocks,
                                 cudaStream_t s);
-// G'_j of the chunk on the box [row0, row0 + nrows) x [col0, col0 + ncols) of the P grid,
-// written (or with accumulate added) to out[(Y - orow0) * opitch + (X - ocol0)].
-cudaError_t launch_reduce_g(const PassArgs& a, float2* out, int j, int row0, int nrows, int col0,
-                            int ncols, int opitch, int orow0, int ocol0, int accumulate,
-                            cudaStream_t s);
+// G'_j of the chunk, every distance in one launch: on the box {row0, rows, col0, cols} of the P
+// grid, written (or with accumulate added) densely to out.
+struct ReduceArgs {
+  float2* out[HOLO_MAX_DIST];
+  int box[HOLO_MAX_DIST][4];
+  int accumulate;
+};
+cudaError_t launch_reduce_g(const PassArgs& a, const ReduceArgs& r, cudaStream_t s);
 cudaError_t launch_ref_residual(const float2* bref, const float* sqrt_dref, long long n2,
                                 float2* rref, double* part, int nblocks, int functional,
                                 cudaStream_t s);
@@ -195,7 +202,13 @@ cudaError_t launch_upsample2(const float2* in, long long count, int N, float2* o
                              cudaStream_t s);
 cudaError_t launch_sum_f64(const double* part, int count, double* out, int accumulate,
                            cudaStream_t s);
-cudaError_t launch_loss_total(double* red, double wref, int acc, int first, cudaStream_t s);
+// d_red of one part of an evaluation: red[0] = the sum of `count` plane partials, red[1] = that of
+// `refcount` reference partials (first part; else kept), and the totals red[3] (running) and
+// red[7] (of the call) of red[0] + wref red[1].
+cudaError_t launch_loss(const double* part, int count, const double* refpart, int refcount,
+                        double* red, double wref, int acc, int first, cudaStream_t s);
+// out[k] = exp(-i pi lambda z f^2) / P, f = k/(P dx), k in [-P/2, P/2) (FP64 arithmetic)
+cudaError_t launch_chirp(float2* out, int P, double lambda, double dx, double z, cudaStream_t s);
 cudaError_t launch_dot(const float2* a, const float2* b, long long n, double* part, int nblocks,
                        cudaStream_t s);
 cudaError_t launch_dot3(const float2* g, const float2* gp, const float2* eta, long long n,
@@ -207,6 +220,5 @@ cudaError_t launch_direction(float2* eta, const float2* g, float beta, long long
                              cudaStream_t s);
 cudaError_t launch_scale_add(float2* out, const float2* in, float alpha, long long n,
                              int accumulate, cudaStream_t s);
-cudaError_t launch_fill_zero(float2* out, long long n, cudaStream_t s);
 
 }  // namespace holo

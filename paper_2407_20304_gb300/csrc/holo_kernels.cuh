@@ -184,10 +184,13 @@ __device__ __forceinline__ void load_chirp_half(float2* dst, const float2* __res
 
 // ------------------------------------------------------------------ generic D-step
 
-// One "FFT -> chirp -> inverse FFT" per line, lines = rows (COLS = false) or columns.
+// One "FFT -> chirp -> inverse FFT" per line, lines = rows (COLS = false) or columns, of every
+// source in turn (block-steps of G lines that never span two sources).  One launch for the J
+// propagations of a probe, or for the sources of its gradient: what they cost at P <= 1024 is
+// launches and half-empty grids (set_probe at P = 256, 4 distances: 9 launches, 55 us).
 template <int P, bool COLS>
 __global__ void __launch_bounds__(COLS ? ColCfg<P>::NT : RowCfg<P>::NT)
-k_line_dstep(LineArgs a, const float2* __restrict__ gtw) {
+k_line_dstep(const __grid_constant__ LineArgs args, const float2* __restrict__ gtw) {
   using L = Line<P>;
   using H = SmemHead<P>;
   using R = RowCfg<P>;
@@ -199,13 +202,20 @@ k_line_dstep(LineArgs a, const float2* __restrict__ gtw) {
   const int t = COLS ? (int)(threadIdx.x / G) : (int)(threadIdx.x % L::T);
   float2* sm = smem + H::WORDS + g * LS;
   L::load_table(smem, gtw);
-  load_chirp_half<P>(chs, a.chirp);
-  __syncthreads();
   const ChirpAt<P> cat(chs, t);
-  const float sg = a.conj_chirp ? -1.f : 1.f;
   auto run = [&](auto sync) HOLO_INLINE {
-    for (int base = blockIdx.x * G; base < a.nlines; base += gridDim.x * G) {
-      const int line = base + g;
+    int s = 0, cur = -1;
+    for (int step = blockIdx.x; step < args.step[args.S]; step += gridDim.x) {
+      while (step >= args.step[s + 1]) ++s;
+      const LineSource& a = args.src[s];
+      if (s != cur) {
+        __syncthreads();
+        load_chirp_half<P>(chs, a.chirp);
+        __syncthreads();
+        cur = s;
+      }
+      const float sg = a.conj_chirp ? -1.f : 1.f;
+      const int line = (step - args.step[s]) * G + g;
       const bool valid = line < a.nlines;
       const float2* in = a.in + (long long)line * a.in_line_stride;
       float2 v[L::E];
@@ -227,12 +237,7 @@ k_line_dstep(LineArgs a, const float2* __restrict__ gtw) {
 #pragma unroll
       for (int c = 0; c < L::E; ++c) {
         const int rel = L::pos(t, c) - a.out_lo;
-        if (valid && (unsigned)rel < (unsigned)a.out_len) {
-          float2* o = out + (long long)rel * a.out_step;
-          float2 r = cscale(v[c], a.alpha);
-          if (a.accumulate) r = cadd(r, *o);
-          *o = r;
-        }
+        if (valid && (unsigned)rel < (unsigned)a.out_len) out[(long long)rel * a.out_step] = v[c];
       }
     }
   };
@@ -1264,15 +1269,18 @@ int multi_blocks(K kernel, int threads, size_t smem, int nitems, int per_sm) {
 }
 
 template <int P, bool COLS>
-cudaError_t launch_lines(const LineArgs& a, const float2* tw, cudaStream_t s) {
+cudaError_t launch_lines(const LineArgs& args, const float2* tw, cudaStream_t s) {
   constexpr int G = COLS ? ColCfg<P>::C : RowCfg<P>::G;
   constexpr int NT = COLS ? ColCfg<P>::NT : RowCfg<P>::NT;
   constexpr size_t SM = COLS ? ColCfg<P>::SMEM_BYTES : RowCfg<P>::SMEM_BYTES;
-  if (a.nlines <= 0) return cudaSuccess;
+  LineArgs a = args;
+  a.step[0] = 0;
+  for (int i = 0; i < a.S; ++i) a.step[i + 1] = a.step[i] + (a.src[i].nlines + G - 1) / G;
+  if (a.step[a.S] <= 0) return cudaSuccess;
   cudaError_t e = cudaFuncSetAttribute(k_line_dstep<P, COLS>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SM);
   if (e != cudaSuccess) return e;
-  const int nb = persistent_blocks(k_line_dstep<P, COLS>, NT, SM, (a.nlines + G - 1) / G);
+  const int nb = persistent_blocks(k_line_dstep<P, COLS>, NT, SM, a.step[a.S]);
   k_line_dstep<P, COLS><<<nb, NT, SM, s>>>(a, tw);
   return cudaGetLastError();
 }
