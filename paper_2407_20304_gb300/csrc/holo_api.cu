@@ -355,18 +355,18 @@ std::vector<float2> chirp_table(int P, double lambda, double dx, double z) {
   return c;
 }
 
-// Twiddle table of one line length (FP64).  P = 2^k, in the layout of holo_line.cuh (E values per
+// Twiddle table of one line length (FP64).  P = 2^k and 3 * 2^k <= 768, in the layout of holo_line.cuh (E values per
 // thread, T = P/E threads, second stage of T2 = min(T, E)): entries [l E + k1] =
 // exp(-2 pi i k1 2^l / (E T2)), l < log2 T2, k1 < E, then for T > E [t] = exp(-2 pi i t / P).
-// P = 3 PB, in the layout of holo_fft.cuh: radix-16 stage s with M(s) = PB/16^(s+1) > 1
+// Larger P = 3 PB, in the layout of holo_fft.cuh: radix-16 stage s with M(s) = PB/16^(s+1) > 1
 // contributes entries [(k-1) M + mu] = exp(-2 pi i mu k 16^s / PB), k = 1..15, then the radix-3
 // step adds exp(-2 pi i r n / P) for r = 1, 2 (outer) and n < PB (inner).
 std::vector<float2> twiddle_table(int P) {
   std::vector<float2> tw;
   const double pi = 3.14159265358979323846;
   auto push = [&](double a) { tw.push_back(make_float2((float)std::cos(a), (float)std::sin(a))); };
-  if (P % 3) {
-    const int E = P >= 512 ? 32 : 16, T = P / E, T2 = std::min(T, E);
+  if (P % 3 || P <= 768) {
+    const int E = P % 3 == 0 ? 48 : (P >= 512 ? 32 : 16), T = P / E, T2 = std::min(T, E);
     for (int m = 1; m < T2; m *= 2)
       for (int k = 0; k < E; ++k) push(-2.0 * pi * (double)k * m / (E * T2));
     if (T > E)

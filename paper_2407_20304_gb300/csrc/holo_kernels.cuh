@@ -53,13 +53,10 @@ struct SmemHead {
 
 // Row passes.  The threads that exchange with one another form a unit: one line of T >= 32
 // threads (two warps at P = 4096, one at 2048 and 1024) or a warp with 32/T lines below; for
-// P = 3 * 2^k, whose T is no multiple of 32, the whole block.  Units of a block share the twiddle
+// P = 1536 and 3072 (whose engine holds block barriers) the whole block.  Units of a block share the twiddle
 // and chirp tables and are otherwise independent: each has its own barrier, so one unit's
 // arithmetic fills the time another spends on its exchange and its loads.
-__host__ __device__ constexpr int r3_row_lines(int T, int g = 0) {
-  return T >= 256 ? 1
-                  : (g == 0 ? r3_row_lines(T, 256 / T) : ((g * T) % 32 ? r3_row_lines(T, g - 1) : g));
-}
+__host__ __device__ constexpr int r3_row_lines(int T) { return T > 128 ? 1 : 256 / T; }
 
 template <int P>
 struct RowCfg {
@@ -72,9 +69,9 @@ struct RowCfg {
   static constexpr int G = NU * GU;  // lines per block
   // line pitch: lines of one half warp on different banks (T < 16 puts several lines in it)
   static constexpr int LS =
-      L::SMEM + (L::R3 ? (P == 192 ? 1 : 0) : (T >= 16 ? 0 : (T == 8 ? 8 : (T == 4 ? 4 : 2))));
+      L::SMEM + (L::R3 ? 0 : (T >= 16 ? 0 : (T == 8 ? 8 : (T == 4 ? 4 : 2))));
   static constexpr size_t SMEM_BYTES = (size_t)(SmemHead<P>::WORDS + G * LS) * sizeof(float2);
-  static constexpr int MINB = L::R3 ? (P == 768 ? 3 : 2) : (P == 4096 ? 1 : (P == 2048 ? 2 : (P >= 512 ? 4 : 6)));
+  static constexpr int MINB = L::R3 ? 2 : (P == 4096 ? 1 : (P == 2048 ? 2 : (L::M3 ? 3 : (P >= 512 ? 4 : 6))));
 };
 
 // Column passes: C adjacent columns interleaved in the lanes, so that one access covers the C
@@ -84,11 +81,11 @@ struct ColCfg {
   using L = Line<P>;
   static constexpr int T = L::T;
   static constexpr int C =
-      L::R3 ? (T >= 192 ? 2 : (T >= 24 ? 4 : (T >= 12 ? 8 : (T >= 6 ? 16 : 32)))) : (P >= 2048 ? 256 : 128) / T;
+      L::R3 ? (T >= 192 ? 2 : 4) : (P >= 2048 ? 256 : 128) / T;
   static constexpr int NT = C * T;
   // line pitch: the C lines' runs in one 128-byte bank row side by side
   static constexpr int EXTRA =
-      L::R3 ? (P == 768 ? 4 : (P == 1536 ? 3 : (P == 96 || P == 192 || P == 384 ? 1 : 0)))
+      L::R3 ? (P == 1536 ? 3 : 0)
             : (C == 2 ? 8 : (C == 4 ? 4 : 2));
   static constexpr int LS = L::SMEM + EXTRA;
   static constexpr size_t SMEM_BYTES = (size_t)(SmemHead<P>::WORDS + C * LS) * sizeof(float2);
@@ -350,11 +347,11 @@ __device__ __forceinline__ void ensure_chirp_key(float2* chs, const float2* __re
   }
 }
 
-// n = P/2 with P = 2^k >= 64: the crop rows and columns P/4 .. 3P/4 are the registers
+// n = P/2 (P = 2^k >= 64, 192, 384, 768): the crop rows and columns P/4 .. 3P/4 are the registers
 // E/4 .. 3E/4 of every thread and the pass-B column groups divide n (HALF forms).
 template <int P>
 __host__ __device__ constexpr bool half_form_ok() {
-  return !Line<P>::R3 && P >= 64;
+  return !Line<P>::R3 && P / 2 % ColCfg<P>::C == 0;
 }
 // c in the middle half of a thread's registers
 template <int P>
@@ -459,7 +456,8 @@ __device__ __forceinline__ void pass_a_step(const PassArgs& a, int s, int next, 
   // E/4 .. 3E/4 hold zeros
   const bool mid = HALF && ((a.mid_x >> j) & 1);
   float2 v[E];
-  constexpr int CH = E / 4 < 8 ? E / 4 : 8;  // the loads of CH registers are issued together
+  // the loads of CH registers (a divisor of E/4) are issued together
+  constexpr int CH = E / 4 < 8 ? E / 4 : (E == 48 ? 6 : 8);
 #pragma unroll
   for (int c0 = 0; c0 < E; c0 += CH) {
     if (HALF && mid && (c0 < E / 4 || c0 >= 3 * E / 4)) {
@@ -617,7 +615,10 @@ __device__ __forceinline__ void pass_c_step(const PassArgs& a, int s, int next, 
     }
   };
   if (HALF && mid)
-    scatter(Idx<E / 4>{}, Idx<E / 2>{});
+    static_for<(E > 32 ? 2 : 1)>([&](auto ic) HOLO_INLINE {
+      constexpr int W = E > 32 ? E / 4 : E / 2;
+      scatter(Idx<E / 4 + W * decltype(ic)::value>{}, Idx<W>{});
+    });
   else
     static_for<E / 8>([&](auto ic) HOLO_INLINE {
       scatter(Idx<8 * decltype(ic)::value>{}, Idx<8>{});
@@ -626,7 +627,7 @@ __device__ __forceinline__ void pass_c_step(const PassArgs& a, int s, int next, 
   // transposed taps of this plane (same FP64-built weights as the forward taps); the buffer
   // holds conj(z).
   const float4* xa = reinterpret_cast<const float4*>(a.xadj + (long long)gp * n);
-  constexpr int EH = HALF ? E / 2 : E, CT = EH < 16 ? EH : 16;
+  constexpr int EH = HALF ? E / 2 : E, CT = EH < 16 ? EH : (E == 48 ? 12 : 16);
 #pragma unroll
   for (int c0 = 0; c0 < EH; c0 += CT) {
     float4 tp[CT];  // (the position's bits, both weights; loaded ahead of the barrier)
@@ -1129,7 +1130,7 @@ __device__ __forceinline__ bool pass_b_run(const PassArgs& a, int bid, int nblk,
 // Registers: two resident blocks of 128 threads may take 255 each; smaller lines need less.
 template <int P>
 constexpr int pass_b_minb() {
-  return Line<P>::R3 ? 1 : (P >= 2048 ? 2 : (P >= 512 ? 4 : 5));
+  return Line<P>::R3 ? 1 : (Line<P>::M3 ? 3 : (P >= 2048 ? 2 : (P >= 512 ? 4 : 5)));
 }
 
 template <int P, bool HALF>

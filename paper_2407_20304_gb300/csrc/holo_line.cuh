@@ -33,11 +33,13 @@
 // the conjugate of the forward transform of the conjugate, and forward and inverse run as two
 // turns of a loop over one copy of the code (17 KB).
 //
-// P = 3 * 2^k: the radix-3 step and the 16-value engine of holo_fft.cuh (E = 16, T = P/16).
+// P = 3 * 2^k, 48 .. 768: the same two stages with E = 48 (stage 1 is 3 x 16 without twiddles).
+// 1536 and 3072 would need 48 rows over 32 or 64 threads: the radix-3 step and the 16-value engine
+// of holo_fft.cuh (E = 16, T = P/16).
 //
-// ZIN (P = 2^k): the inputs outside the middle half P/4 .. 3P/4, i.e. the registers c outside
-// E/4 .. 3E/4, are zero and not read: stage 1's first two levels become 8 additions per 4
-// values, with the same results as zeros passed to the full form.
+// ZIN: the inputs outside the middle half P/4 .. 3P/4, i.e. the registers c outside E/4 .. 3E/4,
+// are zero and not read.  For E = 2^k stage 1's first two levels become 8 additions per 4 values,
+// with the same results as zeros passed to the full form.
 //
 // Synchronisation: every thread of a line calls fft the same number of times; Sync is a barrier
 // over (at least) the threads of the line.  fft starts with a barrier, so the line's buffer may
@@ -174,6 +176,37 @@ __device__ __forceinline__ void dft_const_zin(float2* v) {
   });
 }
 
+// DFT of length 48 as 3 x 16 without twiddles (Good-Thomas: element (16 a + 3 b) mod 48, output k
+// with k mod 3 and k mod 16 the two indices); X[k] is left in v[dft48_at(k)].
+__host__ __device__ constexpr int dft48_at(int k) {
+  return (16 * (k % 3) + 3 * bit_reverse(k % 16, 4)) % 48;
+}
+__device__ __forceinline__ void dft48(float2* v) {
+  static_for<3>([&](auto ac) HOLO_INLINE {
+    constexpr int a = decltype(ac)::value;
+    float2 y[16];
+    static_for<16>([&](auto bc) HOLO_INLINE {
+      constexpr int b = decltype(bc)::value;
+      y[b] = v[(16 * a + 3 * b) % 48];
+    });
+    dft_const_levels<16, 1, 16>(y);
+    static_for<16>([&](auto bc) HOLO_INLINE {
+      constexpr int b = decltype(bc)::value;
+      v[(16 * a + 3 * b) % 48] = y[b];
+    });
+  });
+  const float h = 0.86602540378443865f;  // sqrt(3)/2
+  static_for<16>([&](auto bc) HOLO_INLINE {
+    constexpr int b = decltype(bc)::value;
+    float2 &x0 = v[(3 * b) % 48], &x1 = v[(16 + 3 * b) % 48], &x2 = v[(32 + 3 * b) % 48];
+    const float2 su = cadd(x1, x2), df = csub(x1, x2);
+    const float2 m = make_float2(fmaf(-0.5f, su.x, x0.x), fmaf(-0.5f, su.y, x0.y));
+    x0 = cadd(x0, su);
+    x1 = make_float2(fmaf(h, df.y, m.x), fmaf(-h, df.x, m.y));
+    x2 = make_float2(fmaf(-h, df.y, m.x), fmaf(h, df.x, m.y));
+  });
+}
+
 // DFT of the T values v[S i] w^i (natural order in, X[k] in v[S bit_reverse(k)]), levels M, 2M,
 // ...; tw(l) gives w^{2^l}.
 template <int T, int S, int M, class Tw>
@@ -201,15 +234,20 @@ __device__ __forceinline__ void dft_scaled_levels(float2* v, Tw tw) {
 
 // ------------------------------------------------------------------ lines
 
-template <int P_, bool R3_ = P_ % 3 == 0>
+template <int P_, bool R3_ = (P_ % 3 == 0 && P_ > 768)>
 struct Line;
 
 template <int P_>
 struct Line<P_, false> {
   static constexpr int P = P_;
   static constexpr bool R3 = false;
-  static_assert(is_pow2c(P) && P >= 16 && P <= 4096, "line length");
-  static constexpr int E = P >= 512 ? 32 : 16;
+  static constexpr bool M3 = P % 3 == 0;            // P = 3 * 2^k: E = 48
+  static_assert(is_pow2c(M3 ? P / 3 : P) && P >= 16 && P <= 4096, "line length");
+  static constexpr int E = M3 ? 48 : (P >= 512 ? 32 : 16);
+  // where stage 1 leaves output k
+  __host__ __device__ static constexpr int at(int k) {
+    return M3 ? dft48_at(k) : bit_reverse(k, ilog2c(E));
+  }
   static constexpr int T = P / E;
   static constexpr int R = T > E ? T / E : 1;      // radix of the third stage
   static constexpr int NB = R > 1 ? 1 : E / T;     // second-stage DFTs per thread
@@ -219,7 +257,7 @@ struct Line<P_, false> {
   // every access of a warp is free of bank conflicts.
   static constexpr int RS = R > 1 ? T + 1 : T + 2;
   static constexpr int SMEM = T > 1 ? E * RS : P;  // float2 entries of a line's buffer (>= P)
-  static constexpr int B2 = ilog2c(T2), BE = ilog2c(E);
+  static constexpr int B2 = ilog2c(T2);
   // twiddles: [l][k1] = W_{E T2}^{k1 2^l}, l < log2 T2, then (three stages) [t] = W_P^t
   static constexpr int TAB = E * B2 + (R > 1 ? T : 0);
   static constexpr int TABS = TAB;                 // entries kept in shared memory
@@ -237,14 +275,23 @@ struct Line<P_, false> {
                                              const float2* __restrict__ tab, int t, Sync sync,
                                              bool zin) {
     if constexpr (T > 1) sync();
-    if (ZIN && zin)
-      dft_const_zin<E>(v);
-    else
-      dft_const_levels<E, 1, 4>(v);
-    dft_const_levels<E, 4, E>(v);
+    if constexpr (M3) {
+      if (ZIN && zin) {
+#pragma unroll
+        for (int c = 0; c < E; ++c)
+          if (c < E / 4 || c >= 3 * E / 4) v[c] = make_float2(0.f, 0.f);
+      }
+      dft48(v);
+    } else {
+      if (ZIN && zin)
+        dft_const_zin<E>(v);
+      else
+        dft_const_levels<E, 1, 4>(v);
+      dft_const_levels<E, 4, E>(v);
+    }
     if constexpr (T > 1) {
       static_for<E>([&](auto ic) HOLO_INLINE {
-        constexpr int k = decltype(ic)::value, r = bit_reverse(k, BE);
+        constexpr int k = decltype(ic)::value, r = at(k);
         sm[k * RS + t] = v[r];
       });
       sync();
@@ -267,7 +314,7 @@ struct Line<P_, false> {
       // to natural order (a renaming of registers)
       static_for<E>([&](auto ic) HOLO_INLINE {
         constexpr int c = decltype(ic)::value;
-        constexpr int r = T > 1 ? c % NB + NB * bit_reverse(c / NB, B2) : bit_reverse(c, BE);
+        constexpr int r = T > 1 ? c % NB + NB * bit_reverse(c / NB, B2) : at(c);
         x[c] = v[r];
       });
     } else {
@@ -282,7 +329,7 @@ struct Line<P_, false> {
       dft_scaled_levels<E, 1, 1>(v, [&](int l) HOLO_INLINE { return w2[E * l]; });
       // (the entries a thread writes are those it has read)
       static_for<E>([&](auto ic) HOLO_INLINE {
-        constexpr int k = decltype(ic)::value, r = bit_reverse(k, BE);
+        constexpr int k = decltype(ic)::value, r = at(k);
         own[R * k] = v[r];
       });
       sync();
@@ -310,7 +357,7 @@ struct Line<P_, false> {
 template <int P_>
 struct Line<P_, true> {
   static constexpr int P = P_;
-  static constexpr bool R3 = true;
+  static constexpr bool R3 = true, M3 = true;
   using F = Fft<P>;
   static constexpr int E = 16, T = F::T, SMEM = F::SMEM;
   static constexpr int TAB = F::TW, TABS = F::ROOTS;

@@ -1,4 +1,4 @@
-"""The line transforms of P = 2^k (two or three stages) and the forms built on them.
+"""The line transforms of P = 2^k and 3 * 2^k <= 768 (two or three stages) and the forms built on them.
 
 CPU: a NumPy model of the stages, index for index as the kernels have them, equals the DFT for
 every length, and its shared-memory accesses are free of bank conflicts.  GPU: single propagations
@@ -10,17 +10,17 @@ import pytest
 
 import holo_synth as hs
 
-POW2 = [1 << k for k in range(4, 13)]
+LENGTHS = [1 << k for k in range(4, 13)] + [48, 96, 192, 384, 768]
 
 
 def shape(P):
-    E = 32 if P >= 512 else 16
+    E = 48 if P % 3 == 0 else 32 if P >= 512 else 16
     T = P // E
     R = T // E if T > E else 1
     return E, T, R, (T + 1 if R > 1 else T + 2)
 
 
-@pytest.mark.parametrize("P", POW2)
+@pytest.mark.parametrize("P", LENGTHS)
 def test_stages_equal_the_dft(P):
     E, T, R, _ = shape(P)
     x = np.random.default_rng(P).standard_normal((P, 2)) @ [1, 1j]
@@ -74,7 +74,7 @@ gpu = pytest.mark.gpu
 
 
 @gpu
-@pytest.mark.parametrize("P", POW2)
+@pytest.mark.parametrize("P", LENGTHS)
 def test_propagation_error(P):
     """A transform pair is 2 log2 P levels, each adding about half an ulp (6e-8) of random
     rounding to a value, twice that where 2 a - s carries the error of s: 1.2e-7 sqrt(4 * 12) =
@@ -95,7 +95,8 @@ def test_propagation_error(P):
 
 @gpu
 @pytest.mark.parametrize("n,P", [(30, 64), (32, 64), (64, 128), (66, 128), (128, 256), (256, 512),
-                                 (512, 1024), (510, 1024), (1024, 2048)])
+                                 (512, 1024), (510, 1024), (1024, 2048),
+                                 (24, 48), (48, 96), (96, 192), (192, 384), (384, 768), (386, 768)])
 @pytest.mark.parametrize("shift", [0.0, 0.35])
 def test_gradient_at_the_edges_of_the_half_form(n, P, shift):
     """shift * n pixels move the second angle's boxes out of the middle half."""
