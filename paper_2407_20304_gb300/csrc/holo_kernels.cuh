@@ -64,14 +64,15 @@ struct RowCfg {
   static constexpr int T = L::T;
   static constexpr int GU = L::R3 ? r3_row_lines(T) : (T >= 32 ? 1 : 32 / T);  // lines per unit
   static constexpr int U = GU * T;                                            // threads per unit
-  static constexpr int NU = L::R3 ? 1 : 4;
+  // (at P = 4096 two blocks of two units beat one of four: pass C 8.72 -> 8.41 ms on 393k lines)
+  static constexpr int NU = L::R3 ? 1 : (P == 4096 ? 2 : 4);
   static constexpr int NT = NU * U;
   static constexpr int G = NU * GU;  // lines per block
   // line pitch: lines of one half warp on different banks (T < 16 puts several lines in it)
   static constexpr int LS =
       L::SMEM + (L::R3 ? 0 : (T >= 16 ? 0 : (T == 8 ? 8 : (T == 4 ? 4 : 2))));
   static constexpr size_t SMEM_BYTES = (size_t)(SmemHead<P>::WORDS + G * LS) * sizeof(float2);
-  static constexpr int MINB = L::R3 ? 2 : (P == 4096 ? 1 : (P == 2048 ? 2 : (L::M3 ? 3 : (P >= 512 ? 4 : 6))));
+  static constexpr int MINB = L::R3 ? 2 : (P >= 2048 ? 2 : (L::M3 ? 3 : (P >= 512 ? 4 : 6)));
 };
 
 // Column passes: C adjacent columns interleaved in the lanes, so that one access covers the C
@@ -91,8 +92,15 @@ struct ColCfg {
   static constexpr size_t SMEM_BYTES = (size_t)(SmemHead<P>::WORDS + C * LS) * sizeof(float2);
 };
 
-struct SyncWarp {
-  __device__ __forceinline__ void operator()() const { __syncwarp(); }
+// Column D-steps (no per-thread state besides the line): at P = 4096 four columns and 512 threads,
+// so that every access covers whole 32-byte sectors.
+template <int P>
+struct DColCfg {
+  using L = Line<P>;
+  static constexpr int C = P == 4096 ? 4 : ColCfg<P>::C;
+  static constexpr int NT = C * L::T;
+  static constexpr int LS = P == 4096 ? L::SMEM + 4 : ColCfg<P>::LS;
+  static constexpr size_t SMEM_BYTES = (size_t)(SmemHead<P>::WORDS + C * LS) * sizeof(float2);
 };
 
 // The barrier of a unit of the row passes.
@@ -186,13 +194,13 @@ __device__ __forceinline__ void load_chirp_half(float2* dst, const float2* __res
 // propagations of a probe, or for the sources of its gradient: what they cost at P <= 1024 is
 // launches and half-empty grids (set_probe at P = 256, 4 distances: 9 launches, 55 us).
 template <int P, bool COLS>
-__global__ void __launch_bounds__(COLS ? ColCfg<P>::NT : RowCfg<P>::NT)
+__global__ void __launch_bounds__(COLS ? DColCfg<P>::NT : RowCfg<P>::NT)
 k_line_dstep(const __grid_constant__ LineArgs args, const float2* __restrict__ gtw) {
   using L = Line<P>;
   using H = SmemHead<P>;
   using R = RowCfg<P>;
-  constexpr int G = COLS ? ColCfg<P>::C : R::G;
-  constexpr int LS = COLS ? ColCfg<P>::LS : R::LS;
+  constexpr int G = COLS ? DColCfg<P>::C : R::G;
+  constexpr int LS = COLS ? DColCfg<P>::LS : R::LS;
   extern __shared__ __align__(16) float2 smem[];
   float2* chs = smem + H::TAB;
   const int g = COLS ? (int)(threadIdx.x % G) : (int)(threadIdx.x / L::T);
@@ -213,6 +221,10 @@ k_line_dstep(const __grid_constant__ LineArgs args, const float2* __restrict__ g
       }
       const float sg = a.conj_chirp ? -1.f : 1.f;
       const int line = (step - args.step[s]) * G + g;
+      // a thread group's next row (same source) goes to L2 now
+      if (!COLS && t == 0 && line + (int)gridDim.x * G < a.nlines)
+        l2_prefetch_bulk(a.in + (long long)(line + (int)gridDim.x * G) * a.in_line_stride,
+                         (uint32_t)(a.in_len * sizeof(float2)));
       const bool valid = line < a.nlines;
       const float2* in = a.in + (long long)line * a.in_line_stride;
       float2 v[L::E];
@@ -250,11 +262,11 @@ k_line_dstep(const __grid_constant__ LineArgs args, const float2* __restrict__ g
 // columns at a time, as k_line_dstep's column form.  P = 2^k: turn s < S transforms source s,
 // turn S the conjugate of the sum (one copy of the transform's code, as line_dstep).
 template <int P>
-__global__ void __launch_bounds__(ColCfg<P>::NT)
+__global__ void __launch_bounds__(DColCfg<P>::NT)
 k_cols_sum(const __grid_constant__ SumArgs a, const float2* __restrict__ gtw) {
   using L = Line<P>;
   using H = SmemHead<P>;
-  constexpr int G = ColCfg<P>::C, LS = ColCfg<P>::LS, E = L::E;
+  constexpr int G = DColCfg<P>::C, LS = DColCfg<P>::LS, E = L::E;
   extern __shared__ __align__(16) float2 smem[];
   const int g = threadIdx.x % G, t = threadIdx.x / G;
   float2* sm = smem + H::TAB + g * LS;
@@ -1271,9 +1283,9 @@ int multi_blocks(K kernel, int threads, size_t smem, int nitems, int per_sm) {
 
 template <int P, bool COLS>
 cudaError_t launch_lines(const LineArgs& args, const float2* tw, cudaStream_t s) {
-  constexpr int G = COLS ? ColCfg<P>::C : RowCfg<P>::G;
-  constexpr int NT = COLS ? ColCfg<P>::NT : RowCfg<P>::NT;
-  constexpr size_t SM = COLS ? ColCfg<P>::SMEM_BYTES : RowCfg<P>::SMEM_BYTES;
+  constexpr int G = COLS ? DColCfg<P>::C : RowCfg<P>::G;
+  constexpr int NT = COLS ? DColCfg<P>::NT : RowCfg<P>::NT;
+  constexpr size_t SM = COLS ? DColCfg<P>::SMEM_BYTES : RowCfg<P>::SMEM_BYTES;
   LineArgs a = args;
   a.step[0] = 0;
   for (int i = 0; i < a.S; ++i) a.step[i + 1] = a.step[i] + (a.src[i].nlines + G - 1) / G;
@@ -1357,7 +1369,7 @@ inline int max_sm_smem() {
 
 template <int P>
 cudaError_t launch_cols_sum(const SumArgs& a, const float2* tw, cudaStream_t s) {
-  using Cc = ColCfg<P>;
+  using Cc = DColCfg<P>;
   if (a.S < 1 || a.S > kMaxSumSources) return cudaErrorNotSupported;
   const size_t sm = (size_t)(SmemHead<P>::TAB + Cc::C * Cc::LS) * sizeof(float2);
   cudaError_t e = cudaFuncSetAttribute(k_cols_sum<P>, cudaFuncAttributeMaxDynamicSharedMemorySize,
