@@ -37,6 +37,7 @@ import holo_synth as hs  # noqa: E402
 METRIC = "plane-gradient evals/s at 2048^2 x 4 dist"
 UNIT = "plane-grads/s"
 KERNEL_SOURCES = ("paper_2407_20304_gb300/csrc/holo_kernels.cuh",
+                  "paper_2407_20304_gb300/csrc/holo_line.cuh",
                   "paper_2407_20304_gb300/csrc/holo_fft.cuh")
 FP32_LANES_PER_SM = 128
 
@@ -386,7 +387,7 @@ def run_ours(args, w, rank, world, local_rank):
               "step_frac_balg": round(step_balg / pk["hbm_gbs"], 4),
               "balg_bytes_per_plane": round(sv["total"]),
               "flop_convention": "5 N log2 N per complex FFT of length N plus pointwise flops; "
-                                 "nominal, above a radix-16 FFT's real operation count",
+                                 "nominal, above the transforms' real operation count",
               "peak_source": f"FP32: {sms} SMs x {FP32_LANES_PER_SM} lanes x 2 x {sm_ghz:.3f} GHz "
                              f"({clock_src}); HBM {pk['source']} {pk['hbm_gbs']} GB/s"}
     if alu_frac >= hbm_frac:

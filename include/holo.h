@@ -328,10 +328,9 @@ holo_status holo_set_stream(holo_ctx* ctx, void* stream);
  *   pass_b_stage       pass B's TMA staging of its input tiles: -1 where it fits (default),
  *                      0 off (plain loads), 1 same as -1;
  *   pass_b_split       pass B's last, partial round of column groups: -1 automatic (default:
- *                      split by planes with the plane-split kernel when there are fewer than
- *                      three full rounds), 0 never split (whole column groups per block), 1
- *                      split by the plane-split kernel (no TMA stage), 2 split inside the
- *                      staged kernel, whenever the last round is partial.
+ *                      its planes dealt over all blocks when there are fewer than three full
+ *                      rounds), 0 never split (whole column groups per block), 1 split whenever
+ *                      the last round is partial, without the TMA stage, 2 the same with it.
  * HOLO_ERR_ARG for values outside these ranges. */
 holo_status holo_set_schedule(holo_ctx* ctx, int row_blocks_per_sm, int pass_b_stage,
                               int pass_b_split);

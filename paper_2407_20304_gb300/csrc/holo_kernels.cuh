@@ -12,8 +12,8 @@
 //           detector columns -> Y[box rows][n]
 //   pass B (detector columns): column FFT, chirp, IFFT, keep the n detector rows,
 //           u = ext b + (.), residual r = u - a u/|u| (Eq. gradpsi), loss partial,
-//           r stored for the ext-part of grad_q, then the adjoint column transform
-//           (conjugate chirp) on C* r, keep box rows -> V (in place of Y)
+//           S = sum r kept for the ext-part of grad_q, then the adjoint column transform
+//           on C* r, keep box rows -> conj(V) (in place of Y)
 //   pass C (rows of the box): adjoint row transform -> v on the box columns;
 //           z = conj(p_j) v, x-transpose of the bilinear resample -> h[box rows][n]
 //           (in place of V); conj(w) v -> per-plane buffer for grad_q
@@ -22,11 +22,14 @@
 // All passes run persistent blocks (a grid that fills the GPU once) that load the FFT
 // twiddles into shared memory once and then walk a flat list of work items.
 //
-// Probe shifts s_kj (Eq. min1) use the SHIFT forms of passes A, B and C.  The shift is moved
+// Every propagation D = inverse . chirp . forward of a line is one line_dstep; its adjoint is
+// conj D conj, the chirp being even in frequency.
+//
+// Probe shifts s_kj (Eq. min1) run the passes' general forms with ramps.  The shift is moved
 // off the probe, u_kj = C S_s D_{zhat_j}(p_j * R'_kj psi_k) with R' the resample at object
 // shift t - m~_j s, and S_s D_{zhat_j} is one separable Fourier multiplier: the chirp times
 // the per-plane phase ramps exp(-2 pi i k s / P) of each axis (ramp_x in the row passes,
-// ramp_y in the column pass; conjugated in the adjoints).  The ext-part of the field is then
+// ramp_y in the column pass; at -f for the conjugated adjoints).  The ext-part of the field is then
 // shifted per plane as well, so the box is the whole P x P grid, w holds R' psi itself
 // (ext added back in pass A) and pass B runs with ext = 0 (no b term, T = w_ref r_ref).
 
@@ -52,10 +55,15 @@ struct SmemHead {
 };
 
 // Row passes.  The threads that exchange with one another form a unit: one line of T >= 32
-// threads (two warps at P = 4096, one at 2048 and 1024) or a warp with 32/T lines below; for
-// P = 1536 and 3072 (whose engine holds block barriers) the whole block.  Units of a block share the twiddle
-// and chirp tables and are otherwise independent: each has its own barrier, so one unit's
-// arithmetic fills the time another spends on its exchange and its loads.
+// threads (four warps at P = 4096, two at 2048, one at 1024) or a warp with 32/T lines below; for
+// P = 1536 and 3072 (whose engine holds block barriers) the whole block.  Units of a block share
+// the twiddle and chirp tables and are otherwise independent: each has its own barrier, so one
+// unit's arithmetic fills the time another spends on its exchange and its loads.  What bounds them
+// is the latency of the L2 loads around the transforms at 16 warps per SM (P = 4096: FP32 pipe 45 %
+// and 38 %, shared memory 60 % and 55 % busy in A and C).  393k lines of the 2048^2 chunk: pass A
+// 9.8 -> 7.9 ms, C 9.4 -> 8.4 ms; 512^2, 180 x 4 planes: about 2.1 -> 1.1 ms each.  Units per block
+// (2 at P = 4096, else 4): 4 / 2 / 1 at 4096 took 8.72 / 8.41 / 8.50 ms in pass C, 4 / 2 / 8 at 2048
+// 2.76 / 2.82 / 2.91 ms in pass A.
 __host__ __device__ constexpr int r3_row_lines(int T) { return T > 128 ? 1 : 256 / T; }
 
 template <int P>
@@ -64,7 +72,6 @@ struct RowCfg {
   static constexpr int T = L::T;
   static constexpr int GU = L::R3 ? r3_row_lines(T) : (T >= 32 ? 1 : 32 / T);  // lines per unit
   static constexpr int U = GU * T;                                            // threads per unit
-  // (at P = 4096 two blocks of two units beat one of four: pass C 8.72 -> 8.41 ms on 393k lines)
   static constexpr int NU = L::R3 ? 1 : (P == 4096 ? 2 : 4);
   static constexpr int NT = NU * U;
   static constexpr int G = NU * GU;  // lines per block
@@ -76,7 +83,8 @@ struct RowCfg {
 };
 
 // Column passes: C adjacent columns interleaved in the lanes, so that one access covers the C
-// columns of consecutive rows; for P = 2^k a block is 128 threads, from P = 2048 256.
+// columns of consecutive rows; a block is 128 threads, from P = 2048 256 (P = 4096 with four
+// columns and 512 threads: pass B 18.6 ms against 17.4; P = 1536, 3072: as their T allows).
 template <int P>
 struct ColCfg {
   using L = Line<P>;
@@ -93,7 +101,8 @@ struct ColCfg {
 };
 
 // Column D-steps (no per-thread state besides the line): at P = 4096 four columns and 512 threads,
-// so that every access covers whole 32-byte sectors.
+// so that every access covers whole 32-byte sectors (a 4096^2 propagation 262 -> 214 us, with the
+// row kernel's prefetch).
 template <int P>
 struct DColCfg {
   using L = Line<P>;
@@ -732,7 +741,9 @@ k_rows_multi(const PassArgs* __restrict__ args, const int2* __restrict__ items, 
 
 // Tensor memory of pass B per thread (32-bit columns): b and the residual sum S of its NS crop
 // registers; in the HALF form from P = 1024 also its E chirp entries, so that shared memory holds
-// the blocks that registers allow together with their Y stages.
+// the blocks that registers allow together with their Y stages (the chirp read through L1/L2
+// instead: pass B 19.2 against 17.4 ms on the 2048^2 chunk, 2.97 against 2.77 at 512^2; below P =
+// 1024 neither it nor the stage changed the time).
 template <int P, bool HALF>
 struct PassBMem {
   static constexpr int E = Line<P>::E;
@@ -890,6 +901,13 @@ __device__ __noinline__ void pass_b_next(const PassArgs& a, int bid, int nblk, P
 // Per plane the block runs "column transform, chirp, inverse" twice through one loop body: first
 // on Y, then on the conjugated residual.  The chirp is even in frequency, so the adjoint of D is
 // conj D conj: the second turn yields conj(V), which is what is stored (pass C takes it as is).
+//
+// What bounds it: the transforms themselves (11.7 of 17.4 ms on the 2048^2 chunk of 240 planes, 1.6
+// of 2.8 at 512^2 x 720 planes, alone on the chip), FP32 pipe 48 % and shared memory 51 % busy; the
+// 16-byte pieces of V's stores cost 1.6 ms at P = 4096.  Before (b, S and chirp in shared memory, one
+// block per SM, radix-16 engine): 20.0 and 5.6 ms; 1024^2 x 360 planes 8.9 -> 6.1 ms.  Without the Y
+// stage 22.9 ms.  With the block's work list and descriptors in registers the spills (900 bytes a
+// plane) went to L2: 31.8 ms, so fields are read from shared memory (peek) where they are used.
 //
 // The block's FP64 loss partial goes to a.loss_part[bid].  The caller has loaded the twiddle
 // table at the head of shared memory and, for a staged problem, initialised the Y-stage barrier.

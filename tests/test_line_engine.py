@@ -114,3 +114,21 @@ def test_gradient_at_the_edges_of_the_half_form(n, P, shift):
                                      pr["geo"])
     assert abs(h.forward(psi) - F) / F < 1e-5 and abs(loss - F) / F < 1e-5
     assert rel(gp.cpu().numpy(), gp_ref) < 1e-4 and rel(gq.cpu().numpy(), gq_ref) < 1e-4
+
+
+@gpu
+@pytest.mark.parametrize("n,P,J", [(64, 64, 3), (1024, 1024, 1), (62, 128, 8), (384, 768, 8)])
+def test_gradient_without_padding_and_with_eight_distances(n, P, J):
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    from test_gpu_parity import dev, make_holo, make_problem, rel
+    from oracle import holo as oh
+    z = tuple(4.6e-4 + 0.5e-4 * j for j in range(J))
+    pr = make_problem(n, P, 3, J=J, z=z, seed=5 * n + J, point="object")
+    h = make_holo(pr)
+    loss, gp, gq = h.gradient(dev(pr["psi"], torch.complex64))
+    F, gp_ref, gq_ref = oh.gradients(pr["psi"], pr["q"], pr["t"], pr["sqrt_d"], pr["sqrt_dref"],
+                                     pr["geo"])
+    assert abs(loss - F) / F < 1e-5
+    assert rel(gp.cpu().numpy(), gp_ref) < 1e-4 and rel(gq.cpu().numpy(), gq_ref) < 1e-4
