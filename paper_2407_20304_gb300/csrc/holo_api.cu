@@ -84,7 +84,7 @@ struct holo_ctx {
   double wref = 0.0;
   int functional = HOLO_F2_AMPLITUDE;
   // schedule (holo_set_schedule): row-pass blocks per SM (0: as many as fit), pass-B Y stage
-  // and plane-split form (-1: automatic, 0: off, 1: on where applicable)
+  // and last-round split (-1: automatic, 0: off, 1, 2: on where applicable)
   int sched_row_per_sm = 0, sched_stage = -1, sched_split = -1;
   cudaStream_t stream = nullptr;
   // holo_gradient_host in parts: copy streams and their events (created on first use)
@@ -161,7 +161,7 @@ struct holo_ctx {
   double* d_part = nullptr;
   long long part_cap = 0;
   double* d_dot3 = nullptr;     // partial sums of holo_dy_dots: 3 x (8 x SM count)
-  float2* d_tpart = nullptr;    // pass B (plane-split form): partial residual sums
+  float2* d_tpart = nullptr;    // pass B (split last round): partial residual sums
   size_t tpart_bytes = 0;
   double* d_red = nullptr;      // kRed doubles: loss, reference term, dot, running loss, DY
                                 // dots, call loss; word kErrWord: device-wait error flag
