@@ -79,7 +79,8 @@ constexpr int kErrWord = 8;
 struct holo_ctx {
   holo_geometry geo{};
   int n = 0, P = 0, J = 0, K = 0, chunk = 0;
-  int sms = 1;  // SMs of the context's device
+  int sms = 1;          // SMs of the context's device
+  double line_s = 1.0;  // line_scale(P)
   float ext = 1.f;
   double wref = 0.0;
   int functional = HOLO_F2_AMPLITUDE;
@@ -342,15 +343,42 @@ struct PassTimer {
 };
 
 
-// exp(-i pi lambda z f^2) / P with f = k/(P dx), k in [-P/2, P/2)  (reading of D_z), FP64.
+// The mean factor 1 + d by which a transform of holo_line.cuh scales its values because its
+// constant twiddles are rounded to FP32: |W| of a rounded constant W is 1 + d_W, and a butterfly
+// a +- W b of equally strong a and b scales both by 1 + d_W / 2.  (-7.3e-8 at P = 4096; the four
+// transforms of a plane left u 3e-7 too small, most of its error, and moved the loss twice as
+// much.)  The chirp tables carry the inverse of the two factors of a propagation.
+double line_scale(int P) {
+  if (P % 3 == 0 && P > 768) return 1.0;
+  const int E = P % 3 == 0 ? 16 : (P >= 512 ? 32 : 16), T = P % 3 == 0 ? P / 48 : P / E;
+  const int T2 = std::min(T, E);
+  const double pi = 3.14159265358979323846;
+  auto dev = [&](int j, int n) {  // |W_n^j| - 1 after rounding
+    const double x = (float)std::cos(2.0 * pi * j / n), y = (float)std::sin(2.0 * pi * j / n);
+    return 4 * j % n == 0 ? 0.0 : std::sqrt(x * x + y * y) - 1.0;
+  };
+  double d = 0.0;
+  for (int m = 1; m < E; m *= 2)  // stage 1: the level's m twiddles
+    for (int j = 0; j < m; ++j) d += 0.5 * dev(j, 2 * m) / m;
+  for (int m = 2; m < T2; m *= 2)  // stage 2: m/2 constants (and -i times them) on table entries
+    for (int j = 0; j < m / 2; ++j) d += 0.5 * dev(j, 2 * m) / (m / 2);
+  if (T > E)                       // stage 3: constants W_E^i, squared on the lower level of R = 4
+    for (int i = 0; i < E * E / T; ++i)
+      d += 0.5 * dev(i, E) / (E * E / T) * (T / E == 4 ? 3.0 : 1.0);
+  return 1.0 + d;
+}
+
+// exp(-i pi lambda z f^2) / (P s^2) with f = k/(P dx), k in [-P/2, P/2)  (reading of D_z) and s the
+// transforms' scale, FP64.
 std::vector<float2> chirp_table(int P, double lambda, double dx, double z) {
   std::vector<float2> c(P);
+  const double s = line_scale(P), scale = 1.0 / (P * s * s);
   const double pi = 3.14159265358979323846;
   for (int k = 0; k < P; ++k) {
     const double kk = k < P / 2 ? k : k - P;
     const double f = kk / (P * dx);
     const double ph = -pi * lambda * z * f * f;
-    c[k] = make_float2((float)(std::cos(ph) / P), (float)(std::sin(ph) / P));
+    c[k] = make_float2((float)(std::cos(ph) * scale), (float)(std::sin(ph) * scale));
   }
   return c;
 }
@@ -903,6 +931,7 @@ holo_status holo_create(const holo_geometry* geo, void* stream, holo_ctx** out) 
   c->wref = geo->w_ref;
   c->stream = (cudaStream_t)stream;
   c->ops = ops;
+  c->line_s = line_scale(P);
   {
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess ||
@@ -1483,7 +1512,7 @@ holo_status holo_propagate(holo_ctx* c, const void* in, void* out, double z) {
   // the chirp is made on the device: at P = 4096 the host's table, its copy and the wait for it
   // took 100 of 265 us
   HOLO_LAUNCH(c, holo::launch_chirp(c->d_chirp_tmp, c->P, c->geo.wavelength, c->geo.pixel, z,
-                                    c->stream));
+                                    1.0 / (c->P * c->line_s * c->line_s), c->stream));
   return dstep2d(c, (const float2*)in, (float2*)out, c->d_chirp_tmp, 0);
 }
 

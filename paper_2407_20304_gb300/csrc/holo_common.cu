@@ -333,7 +333,8 @@ __global__ void k_loss(const double* __restrict__ part, int count,
 }
 
 // The chirp table of one distance (FP64; entry k at frequency k/(P dx), k in [-P/2, P/2)).
-__global__ void k_chirp(float2* __restrict__ out, int P, double lambda, double dx, double z) {
+__global__ void k_chirp(float2* __restrict__ out, int P, double lambda, double dx, double z,
+                        double scale) {
   const int k = blockIdx.x * blockDim.x + threadIdx.x;
   if (k >= P) return;
   const double kk = k < P / 2 ? k : k - P;
@@ -341,7 +342,7 @@ __global__ void k_chirp(float2* __restrict__ out, int P, double lambda, double d
   const double ph = -3.14159265358979323846 * lambda * z * f * f;
   double sn, cs;
   sincos(ph, &sn, &cs);
-  out[k] = make_float2((float)(cs / P), (float)(sn / P));
+  out[k] = make_float2((float)(cs * scale), (float)(sn * scale));
 }
 
 // The vector kernels run on float2 (one complex) or, where every pointer lies on a 16-byte boundary
@@ -596,8 +597,9 @@ cudaError_t launch_loss(const double* part, int count, const double* refpart, in
   return cudaGetLastError();
 }
 
-cudaError_t launch_chirp(float2* out, int P, double lambda, double dx, double z, cudaStream_t s) {
-  k_chirp<<<(P + 63) / 64, 64, 0, s>>>(out, P, lambda, dx, z);
+cudaError_t launch_chirp(float2* out, int P, double lambda, double dx, double z, double scale,
+                         cudaStream_t s) {
+  k_chirp<<<(P + 63) / 64, 64, 0, s>>>(out, P, lambda, dx, z, scale);
   return cudaGetLastError();
 }
 

@@ -207,8 +207,9 @@ cudaError_t launch_sum_f64(const double* part, int count, double* out, int accum
 // red[7] (of the call) of red[0] + wref red[1].
 cudaError_t launch_loss(const double* part, int count, const double* refpart, int refcount,
                         double* red, double wref, int acc, int first, cudaStream_t s);
-// out[k] = exp(-i pi lambda z f^2) / P, f = k/(P dx), k in [-P/2, P/2) (FP64 arithmetic)
-cudaError_t launch_chirp(float2* out, int P, double lambda, double dx, double z, cudaStream_t s);
+// out[k] = scale exp(-i pi lambda z f^2), f = k/(P dx), k in [-P/2, P/2) (FP64 arithmetic)
+cudaError_t launch_chirp(float2* out, int P, double lambda, double dx, double z, double scale,
+                         cudaStream_t s);
 cudaError_t launch_dot(const float2* a, const float2* b, long long n, double* part, int nblocks,
                        cudaStream_t s);
 cudaError_t launch_dot3(const float2* g, const float2* gp, const float2* eta, long long n,
