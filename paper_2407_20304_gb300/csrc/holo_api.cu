@@ -15,6 +15,7 @@
 
 #include "holo.h"
 #include "holo_internal.h"
+#include "holo_split.h"
 
 namespace holo {
 const Ops* ops_16();
@@ -597,12 +598,11 @@ PassArgs pass_args(holo_ctx* c, int k0, int nk, const void* psi) {
 //                T = ext sum_kj r_kj (+ w_ref r_ref on the first part);
 //   eval_qgrad:  grad_q of the whole chunk from T and the per-plane conj(w) v.
 // Pass B's grid.  Whole column groups go to the blocks in rounds.  When that leaves a partial
-// last round, the (group, plane) items of that round can be spread over all blocks (pb_split 1:
-// without the Y stage, 2: with it where it fits; automatic when there are fewer than three full
-// rounds, i.e. small n: at n = 2048, 1024 groups on 304 blocks, the whole-group form takes 17.4 ms
-// and the split 18.1, the few busy blocks of the last round running faster than a full one).  A
-// block of a split gets at least two planes (128^2, 8 x 4 planes: 44 us, with one plane 56 us, with
-// four 46 us).  The partial residual sums of a split need tslots slots of [n][C] per block.
+// last round, the (group, plane) items of that round can be spread over all blocks (holo_split.h;
+// pb_split 1: without the Y stage, 2: with it where it fits; automatic when there are fewer than
+// three full rounds, i.e. small n: at n = 2048, 1024 groups on 304 blocks, the whole-group form takes
+// 17.4 ms and the split 18.1, the few busy blocks of the last round running faster than a full one).
+// The partial residual sums of a split need tslots slots of [n][C] per block.
 holo_status pass_b_grid(holo_ctx* c, PassArgs& a, bool gradient, int* nblocks) {
   const int groups = a.pass_b_items;
   const int half = c->ops->half_form(c->n, c->probe_shift);
@@ -619,10 +619,8 @@ holo_status pass_b_grid(holo_ctx* c, PassArgs& a, bool gradient, int* nblocks) {
     return HOLO_OK;
   }
   const long long per = (long long)a.J * a.nk;
-  const int nbx = (int)std::min((long long)full, std::max((long long)c->sms, groups * per / 2));
-  const long long rounds = groups / nbx, tail = groups - rounds * nbx, titems = tail * per;
-  const long long range = (titems + nbx - 1) / nbx;
-  a.tslots = titems > 0 ? (int)((range + per - 1) / per + 1) : 0;
+  const int nbx = holo::split_blocks(full, c->sms, groups * per);
+  a.tslots = holo::split_slots((groups % nbx) * per, nbx, per);
   *nblocks = nbx;
   if (!gradient) return HOLO_OK;
   const size_t need = sizeof(float2) * (size_t)nbx * a.tslots * c->n * c->ops->pass_b_cols;
