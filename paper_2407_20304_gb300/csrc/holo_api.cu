@@ -606,13 +606,12 @@ PassArgs pass_args(holo_ctx* c, int k0, int nk, const void* psi) {
 holo_status pass_b_grid(holo_ctx* c, PassArgs& a, bool gradient, int* nblocks) {
   const int groups = a.pass_b_items;
   const int half = c->ops->half_form(c->n, c->probe_shift);
-  if (c->sched_split == 1) a.ymap = nullptr;
-  const int full = c->ops->pass_b_blocks(1 << 30, half, a.ymap ? a.max_box_rows : 0);
-  const bool partial = groups % full != 0;
-  if (c->sched_split < 0)
-    a.pb_split = partial && groups / full < 3 ? 2 : 0;
-  else
-    a.pb_split = partial ? c->sched_split : 0;
+  int full = c->ops->pass_b_blocks(1 << 30, half, a.ymap ? a.max_box_rows : 0);
+  a.pb_split = holo::split_form(c->sched_split, groups, full);
+  if (a.pb_split == 1 && a.ymap) {
+    a.ymap = nullptr;
+    full = c->ops->pass_b_blocks(1 << 30, half, 0);
+  }
   a.tslots = 0;
   if (!a.pb_split) {
     *nblocks = std::min(full, groups);

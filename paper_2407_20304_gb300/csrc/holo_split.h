@@ -28,6 +28,15 @@ HOLO_SPLIT_FN int split_blocks(int full, int sms, long long items) {
   return (int)(b < 1 ? 1 : b);
 }
 
+// The form of pass B's last round: 0 whole groups, 1 split without the Y stage, 2 split with it.
+// sched: what the user asked for (-1 automatic).  With full rounds only there is nothing to split,
+// whatever was asked for, and the stage stays.
+HOLO_SPLIT_FN int split_form(int sched, int groups, int full) {
+  if (groups % full == 0) return 0;
+  if (sched >= 0) return sched;
+  return groups / full < 3 ? 2 : 0;
+}
+
 // First item of block b.
 HOLO_SPLIT_FN long long split_begin(long long titems, int nblk, int b) { return titems * b / nblk; }
 

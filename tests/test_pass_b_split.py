@@ -16,6 +16,7 @@ CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))),
 WRAP = """
 #include "holo_split.h"
 extern "C" {
+int form(int sched, int groups, int full) { return holo::split_form(sched, groups, full); }
 int blocks(int full, int sms, long long items) { return holo::split_blocks(full, sms, items); }
 long long begin(long long t, int nblk, int b) { return holo::split_begin(t, nblk, b); }
 int slots(long long t, int nblk, long long per) { return holo::split_slots(t, nblk, per); }
@@ -55,6 +56,16 @@ def test_blocks_follow_the_items(rules, full):
         # only where every SM already has two blocks
         assert b >= min(items, 152)
         assert b == min(full, items) or b >= min(full, 304)
+
+
+@pytest.mark.parametrize("full", [152, 304, 608])
+def test_full_rounds_are_never_split(rules, full):
+    """Form 1 gives up the Y stage: it must not be taken where no round is partial."""
+    for sched in (-1, 0, 1, 2):
+        for rounds in (1, 2, 5):
+            assert rules.form(sched, rounds * full, full) == 0
+            partial = rules.form(sched, rounds * full + 1, full)
+            assert partial == (sched if sched >= 0 else (2 if rounds < 3 else 0))
 
 
 @pytest.mark.parametrize("groups,per", [(1, 1), (1, 2), (1, 7), (1, 40), (2, 8), (5, 3), (13, 20),
