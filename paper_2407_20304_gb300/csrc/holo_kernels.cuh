@@ -1061,6 +1061,9 @@ __device__ __forceinline__ bool pass_b_run(const PassArgs& a, int bid, int nblk,
           a.dblk +
           (((long long)(a.k0 - a.data_k0) * a.J + lp) * a.dgroups + cg) * (long long)n * C + g;
       float2* uo = a.u_out ? a.u_out + (long long)lp * n * n + col : nullptr;
+      // The plane's loss terms of the thread: FP32 over groups of four, the groups added in FP32, FP64
+      // from there on.  A term meets 3 + NS/4 - 1 roundings at most (6 at NS = 16, 10 at 32, 14 at 48);
+      // one chain over all NS would meet NS - 1.
       float lsum = 0.f;
       // (every load of the crop rows' data is issued before the first use)
       float dat[NS];
@@ -1073,6 +1076,7 @@ __device__ __forceinline__ bool pass_b_run(const PassArgs& a, int bid, int nblk,
       for (int k = 0; k < NS; k += 4) {
         float2 b[4], S[4];
         tmem_load4x2(b, S, tm + 2 * k, tm + 2 * NS + 2 * k);
+        float l4 = 0.f;
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
           const int c = S0 + k + i;
@@ -1094,13 +1098,14 @@ __device__ __forceinline__ bool pass_b_run(const PassArgs& a, int bid, int nblk,
               diff = mag - dat[k + i];
               f = mag > 0.f ? 1.f - __fdividef(dat[k + i], mag) : 0.f;
             }
-            lsum = fmaf(diff, diff, lsum);
+            l4 = fmaf(diff, diff, l4);
             if (uo) uo[(long long)rr * n] = u;
             r = cscale(u, f);
           }
           S[i] = cadd(S[i], r);
           v[c] = cconj(r);
         }
+        lsum += l4;
         if (a.adj) tmem_store4(tm + 2 * NS + 2 * k, S);
       }
       dsum += (double)lsum;
