@@ -448,7 +448,7 @@ __device__ __forceinline__ void pass_a_step(const PassArgs& a, int s, int next, 
 #pragma unroll 8
       for (int c = 0; c < E / 2; ++c) mix(t + L::T * c);
     } else {
-#pragma unroll 4
+#pragma unroll 8
       for (int ix = t; ix < n; ix += L::T) mix(ix);
     }
   }
@@ -478,8 +478,9 @@ __device__ __forceinline__ void pass_a_step(const PassArgs& a, int s, int next, 
   // E/4 .. 3E/4 hold zeros
   const bool mid = HALF && ((a.mid_x >> j) & 1);
   float2 v[E];
-  // the loads of CH registers (a divisor of E/4) are issued together
-  constexpr int CH = E / 4 < 8 ? E / 4 : (E == 48 ? 6 : 8);
+  // the loads of CH registers (a divisor of E/4) are issued together (E = 48: 12 take 372 us where 6
+  // took 409, 768^2 on 768^2, 24 x 3 planes)
+  constexpr int CH = E == 48 ? 12 : (E / 4 < 8 ? E / 4 : 8);
 #pragma unroll
   for (int c0 = 0; c0 < E; c0 += CH) {
     if (HALF && mid && (c0 < E / 4 || c0 >= 3 * E / 4)) {
@@ -773,6 +774,11 @@ size_t pass_b_smem(int srows = 0) {
   return srows > 0 ? base + 128 + pass_b_stage_bytes<P>(srows) : base;
 }
 
+// Crop rows per run of pass B's loads of b and of the data (a divisor of NS, a multiple of 4).
+__host__ __device__ constexpr int crop_run(int ns) {
+  return ns % 16 == 0 ? 16 : (ns % 12 == 0 ? 12 : 8);
+}
+
 // One plane of a block's pass-B work, in shared memory: the block's threads read a field where
 // they need it, so that no register holds it through the transforms.
 struct PassBPlane {
@@ -949,19 +955,25 @@ __device__ __forceinline__ bool pass_b_run(const PassArgs& a, int bid, int nblk,
     if (peek(pl.first)) {
       // (the stores and loads of tensor memory take whole warps)
       const int col = peek(pl.cg) * C + g;
+      // (RUN loads in flight: four at a time the twelve rounds of NS = 48 took 5 us of a small problem)
+      constexpr int RUN = crop_run(NS);
 #pragma unroll 1
-      for (int k = 0; k < NS; k += 4) {
-        float2 x[4], zero[4];
+      for (int k = 0; k < NS; k += RUN) {
+        float2 x[RUN / 4][4], zero[4];
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
+        for (int i = 0; i < 4; ++i) zero[i] = make_float2(0.f, 0.f);
+#pragma unroll
+        for (int i = 0; i < RUN; ++i) {
           const int rr = L::pos(t, S0 + k + i) - lo;
-          zero[i] = make_float2(0.f, 0.f);
-          x[i] = (col < n && (unsigned)rr < (unsigned)n && ext != 0.f)
-                     ? __ldg(a.bref + (long long)rr * n + col)
-                     : zero[i];
+          x[i / 4][i % 4] = (col < n && (unsigned)rr < (unsigned)n && ext != 0.f)
+                                ? __ldg(a.bref + (long long)rr * n + col)
+                                : make_float2(0.f, 0.f);
         }
-        tmem_store4(tm + 2 * k, x);
-        tmem_store4(tm + 2 * NS + 2 * k, zero);
+#pragma unroll
+        for (int i = 0; i < RUN; i += 4) {
+          tmem_store4(tm + 2 * (k + i), x[i / 4]);
+          tmem_store4(tm + 2 * NS + 2 * (k + i), zero);
+        }
       }
       tmem_store_done();
     }
@@ -971,11 +983,12 @@ __device__ __forceinline__ bool pass_b_run(const PassArgs& a, int bid, int nblk,
         if (pkey * 16 + j != jcur) {
           const float2* chg = a.chirp_zhat + (long long)j * P;
 #pragma unroll 1
-          for (int k = 0; k < E; k += 4) {
-            float2 x[4];
+          for (int k = 0; k < E; k += 16) {
+            float2 x[4][4];
 #pragma unroll
-            for (int i = 0; i < 4; ++i) x[i] = __ldg(chg + L::fpos(t, k + i));
-            tmem_store4(tm + 4 * NS + 2 * k, x);
+            for (int i = 0; i < 16; ++i) x[i / 4][i % 4] = __ldg(chg + L::fpos(t, k + i));
+#pragma unroll
+            for (int i = 0; i < 4; ++i) tmem_store4(tm + 4 * NS + 2 * (k + 4 * i), x[i]);
           }
           tmem_store_done();
           jcur = pkey * 16 + j;
@@ -1065,48 +1078,53 @@ __device__ __forceinline__ bool pass_b_run(const PassArgs& a, int bid, int nblk,
       // from there on.  A term meets 3 + NS/4 - 1 roundings at most (6 at NS = 16, 10 at 32, 14 at 48);
       // one chain over all NS would meet NS - 1.
       float lsum = 0.f;
-      // (every load of the crop rows' data is issued before the first use)
-      float dat[NS];
+      // (the loads of RUN crop rows' data are issued together, ahead of their use; all NS at once
+      // spill at NS = 32 and 48)
+      constexpr int RUN = crop_run(NS);
 #pragma unroll
-      for (int k = 0; k < NS; ++k) {
-        const int rr = L::pos(t, S0 + k) - lo;
-        dat[k] = (HALF || (valid && (unsigned)rr < (unsigned)n)) ? __ldg(ad + rr * C) : 0.f;
-      }
+      for (int k0 = 0; k0 < NS; k0 += RUN) {
+        float dat[RUN];
 #pragma unroll
-      for (int k = 0; k < NS; k += 4) {
-        float2 b[4], S[4];
-        tmem_load4x2(b, S, tm + 2 * k, tm + 2 * NS + 2 * k);
-        float l4 = 0.f;
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          const int c = S0 + k + i;
-          const int rr = L::pos(t, c) - lo;
-          float2 r = make_float2(0.f, 0.f);
-          if (HALF || (valid && (unsigned)rr < (unsigned)n)) {
-            float2 u = v[c];
-            u.x = fmaf(ext, b[i].x, u.x);
-            u.y = fmaf(ext, b[i].y, u.y);
-            const float i2 = fmaf(u.x, u.x, u.y * u.y);
-            // F2: (|u| - a)^2, r = u - a u/|u| (u/|u| := 0 at |u| = 0);
-            // F1: (|u|^2 - d)^2, r = 2 (|u|^2 - d) u
-            float diff, f;
-            if (a.functional) {
-              diff = i2 - dat[k + i];
-              f = 2.f * diff;
-            } else {
-              const float mag = sqrtf(i2);
-              diff = mag - dat[k + i];
-              f = mag > 0.f ? 1.f - __fdividef(dat[k + i], mag) : 0.f;
-            }
-            l4 = fmaf(diff, diff, l4);
-            if (uo) uo[(long long)rr * n] = u;
-            r = cscale(u, f);
-          }
-          S[i] = cadd(S[i], r);
-          v[c] = cconj(r);
+        for (int k = 0; k < RUN; ++k) {
+          const int rr = L::pos(t, S0 + k0 + k) - lo;
+          dat[k] = (HALF || (valid && (unsigned)rr < (unsigned)n)) ? __ldg(ad + rr * C) : 0.f;
         }
-        lsum += l4;
-        if (a.adj) tmem_store4(tm + 2 * NS + 2 * k, S);
+#pragma unroll
+        for (int k = 0; k < RUN; k += 4) {
+          float2 b[4], S[4];
+          tmem_load4x2(b, S, tm + 2 * (k0 + k), tm + 2 * NS + 2 * (k0 + k));
+          float l4 = 0.f;
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            const int c = S0 + k0 + k + i;
+            const int rr = L::pos(t, c) - lo;
+            float2 r = make_float2(0.f, 0.f);
+            if (HALF || (valid && (unsigned)rr < (unsigned)n)) {
+              float2 u = v[c];
+              u.x = fmaf(ext, b[i].x, u.x);
+              u.y = fmaf(ext, b[i].y, u.y);
+              const float i2 = fmaf(u.x, u.x, u.y * u.y);
+              // F2: (|u| - a)^2, r = u - a u/|u| (u/|u| := 0 at |u| = 0);
+              // F1: (|u|^2 - d)^2, r = 2 (|u|^2 - d) u
+              float diff, f;
+              if (a.functional) {
+                diff = i2 - dat[k + i];
+                f = 2.f * diff;
+              } else {
+                const float mag = sqrtf(i2);
+                diff = mag - dat[k + i];
+                f = mag > 0.f ? 1.f - __fdividef(dat[k + i], mag) : 0.f;
+              }
+              l4 = fmaf(diff, diff, l4);
+              if (uo) uo[(long long)rr * n] = u;
+              r = cscale(u, f);
+            }
+            S[i] = cadd(S[i], r);
+            v[c] = cconj(r);
+          }
+          lsum += l4;
+          if (a.adj) tmem_store4(tm + 2 * NS + 2 * (k0 + k), S);
+        }
       }
       dsum += (double)lsum;
       if (!a.adj) break;
@@ -1163,15 +1181,22 @@ __device__ __forceinline__ bool pass_b_run(const PassArgs& a, int bid, int nblk,
   return true;
 }
 
-// Registers: two resident blocks of 128 threads may take 255 each; smaller lines need less.
-template <int P>
+// Resident blocks that the registers must allow, hence the registers a thread may take: 128 at two
+// blocks of 256 threads (P = 2048, 4096) or four of 128 (512, 1024), 96 at five (up to 256), 168 at
+// three (3 * 2^k, n = P/2 form) and 255 at two (its general form, whose b and S leave room for two
+// blocks in tensor memory: with the bound at three it kept to 168 registers and spilled 550 bytes, but
+// two blocks ran all the same; 768^2 on 768^2, 24 x 3 planes: 1330 -> 710 us).  P = 1536 and 3072: one
+// block of 384 threads.
+template <int P, bool HALF>
 constexpr int pass_b_minb() {
-  return Line<P>::R3 ? 1 : (Line<P>::M3 ? 3 : (P >= 2048 ? 2 : (P >= 512 ? 4 : 5)));
+  using L = Line<P>;
+  constexpr int b = L::R3 ? 1 : (L::M3 ? 3 : (P >= 2048 ? 2 : (P >= 512 ? 4 : 5)));
+  return b < PassBMem<P, HALF>::MAXB ? b : PassBMem<P, HALF>::MAXB;
 }
 
 template <int P, bool HALF>
-__global__ void __launch_bounds__(ColCfg<P>::NT, pass_b_minb<P>())
-k_pass_b(const __grid_constant__ PassArgs a) {
+__global__ void __launch_bounds__(ColCfg<P>::NT, pass_b_minb<P, HALF>())
+k_pass_b(const __grid_constant__ PassArgs args) {
   extern __shared__ __align__(16) float2 smem[];
   __shared__ double red[32];
   __shared__ uint64_t ybar;
@@ -1179,6 +1204,19 @@ k_pass_b(const __grid_constant__ PassArgs a) {
   __shared__ PassBState state;
   using M = PassBMem<P, HALF>;
   if (threadIdx.x < 32) tmem_alloc(&tbase, M::COLS);
+  // Up to P = 768 the loops read the arguments from shared memory: constant-bank values that do not
+  // change are kept in registers or make the compiler copy the loops (at 96 to 168 registers 20 to 550
+  // bytes of spills, from shared memory none up to 256 and half at 512; 384^2 on 768^2 206 -> 195 us,
+  // 258^2 on 512^2, 24 x 3 planes, 116 -> 107 us).  Longer lines lose by it (512^2 on 1024^2 411 ->
+  // 434 us, 2048^2 on 4096^2 2395 -> 2472 us).
+  constexpr bool ARGS_SHARED = P <= 768;
+  __shared__ PassArgs sargs;
+  const PassArgs& a = ARGS_SHARED ? sargs : args;
+  if (ARGS_SHARED) {
+    for (int i = threadIdx.x; i < (int)(sizeof(PassArgs) / sizeof(int)); i += blockDim.x)
+      reinterpret_cast<int*>(&sargs)[i] = reinterpret_cast<const int*>(&args)[i];
+    __syncthreads();
+  }
   Line<P>::load_table(smem, a.twiddles);
   if (threadIdx.x == 0) mbar_init(&ybar);
   __syncthreads();
@@ -1194,7 +1232,7 @@ k_pass_b(const __grid_constant__ PassArgs a) {
 // every problem's results (loss partials included) are those of its own launch bit for bit.
 // A Y-stage wait that gives up sets the error word of every problem of the launch.
 template <int P, bool HALF>
-__global__ void __launch_bounds__(ColCfg<P>::NT, pass_b_minb<P>())
+__global__ void __launch_bounds__(ColCfg<P>::NT, pass_b_minb<P, HALF>())
 k_pass_b_multi(const PassArgs* __restrict__ args, const int2* __restrict__ items, int nitems,
                int nprob) {
   extern __shared__ __align__(16) float2 smem[];
