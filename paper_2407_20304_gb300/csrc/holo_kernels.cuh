@@ -36,6 +36,7 @@
 #pragma once
 
 #include <algorithm>
+#include <atomic>
 #include <type_traits>
 
 #include "holo_internal.h"
@@ -745,17 +746,21 @@ k_rows_multi(const PassArgs* __restrict__ args, const int2* __restrict__ items, 
 // registers; in the HALF form from P = 1024 also its E chirp entries, so that shared memory holds
 // the blocks that registers allow together with their Y stages (the chirp read through L1/L2
 // instead: pass B 19.2 against 17.4 ms on the 2048^2 chunk, 2.97 against 2.77 at 512^2; below P =
-// 1024 neither it nor the stage changed the time).
+// 1024 neither it nor the stage changed the time).  The general forms of these lengths have no room
+// for it there; their chirp is in shared memory unless the Y stage fits only without it, then it is
+// read through L1/L2 (see pass_b_chirp_global).
 template <int P, bool HALF>
 struct PassBMem {
   static constexpr int E = Line<P>::E;
   static constexpr int NS = HALF ? E / 2 : E;
   static constexpr bool CHIRP_TM = HALF && P >= 1024;
+  static constexpr bool CHIRP_ANY = !HALF && P >= 1024 && !Line<P>::R3;
   static constexpr int WORDS = 4 * NS + (CHIRP_TM ? 2 * E : 0);
   static constexpr int COLS = tmem_pow2(WORDS * ((ColCfg<P>::NT + 127) / 128));
   static_assert(COLS <= 512, "tensor memory");
   static constexpr int MAXB = 512 / COLS;  // resident blocks per SM
-  static constexpr int HEAD = CHIRP_TM ? SmemHead<P>::TAB : SmemHead<P>::WORDS;
+  // in front of the exchange lines: twiddles, and the chirp unless it has a place of its own
+  static constexpr int HEAD = CHIRP_TM || CHIRP_ANY ? SmemHead<P>::TAB : SmemHead<P>::WORDS;
 };
 
 // Y stage of pass B: whole TMA boxes covering `rows` box rows of C columns.
@@ -765,12 +770,13 @@ size_t pass_b_stage_bytes(int rows) {
   return (size_t)((rows + BOX - 1) / BOX) * BOX * ColCfg<P>::C * sizeof(float2);
 }
 
-// Shared memory of pass B: head, C exchange lines; with srows > 0 also the Y stage for planes of
-// up to srows box rows (128-byte aligned).
+// Shared memory of pass B: head, C exchange lines, with CHIRP_ANY the chirp unless chirp_global; with
+// srows > 0 also the Y stage for planes of up to srows box rows (128-byte aligned).
 template <int P, bool HALF>
-size_t pass_b_smem(int srows = 0) {
-  const size_t base =
-      (size_t)(PassBMem<P, HALF>::HEAD + ColCfg<P>::C * ColCfg<P>::LS) * sizeof(float2);
+size_t pass_b_smem(int srows, bool chirp_global) {
+  using M = PassBMem<P, HALF>;
+  const int chirp = M::CHIRP_ANY && !chirp_global ? SmemHead<P>::CHIRP : 0;
+  const size_t base = (size_t)(M::HEAD + ColCfg<P>::C * ColCfg<P>::LS + chirp) * sizeof(float2);
   return srows > 0 ? base + 128 + pass_b_stage_bytes<P>(srows) : base;
 }
 
@@ -918,22 +924,23 @@ __device__ __noinline__ void pass_b_next(const PassArgs& a, int bid, int nblk, P
 //
 // The block's FP64 loss partial goes to a.loss_part[bid].  The caller has loaded the twiddle
 // table at the head of shared memory and, for a staged problem, initialised the Y-stage barrier.
-// The resident chirp table is identified by pkey * 16 + distance.  Returns false when a bounded
-// Y-stage wait gave up (the problem's error word is then set).
+// The resident chirp table is identified by pkey * 16 + distance; chirp_global (CHIRP_ANY only, one
+// value for the whole launch): there is none, its entries are read from global memory.  Returns false
+// when a bounded Y-stage wait gave up (the problem's error word is then set).
 template <int P, bool HALF>
 __device__ __forceinline__ bool pass_b_run(const PassArgs& a, int bid, int nblk, float2* smem,
                                            uint32_t tmem, double* red, uint64_t* ybarp,
                                            PassBState& st, uint32_t& yphase, int pkey,
-                                           int& jcur) {
+                                           int& jcur, bool chirp_global) {
   using L = Line<P>;
   using Cc = ColCfg<P>;
   using H = SmemHead<P>;
   using M = PassBMem<P, HALF>;
   constexpr int C = Cc::C, E = L::E, NS = M::NS, S0 = HALF ? E / 4 : 0;
   static_assert(!HALF || half_form_ok<P>(), "HALF form");
-  float2* chs = smem + H::TAB;
+  chirp_global = M::CHIRP_ANY && chirp_global;
+  float2* chs = smem + (M::CHIRP_ANY ? M::HEAD + C * Cc::LS : H::TAB);
   const int g = threadIdx.x % C, t = threadIdx.x / C;
-  const ChirpAt<P> cat(chs, t);
   float2* sm = smem + M::HEAD + g * Cc::LS;
   const uint32_t tm = tmem_own(tmem, M::WORDS);
   const int n = a.n, lo = P / 2 - n / 2;
@@ -942,8 +949,9 @@ __device__ __forceinline__ bool pass_b_run(const PassArgs& a, int bid, int nblk,
   double dsum = 0.0;
   // Y stage: the tile of the block's next plane is in flight while the current one computes
   // (aligned at run time: the dynamic shared memory of a block starts on a 16-byte boundary only)
-  float2* stg = reinterpret_cast<float2*>(
-      (reinterpret_cast<uintptr_t>(smem + M::HEAD + C * Cc::LS) + 127) & ~static_cast<uintptr_t>(127));
+  float2* const end = smem + M::HEAD + C * Cc::LS + (M::CHIRP_ANY && !chirp_global ? H::CHIRP : 0);
+  float2* stg = reinterpret_cast<float2*>((reinterpret_cast<uintptr_t>(end) + 127) &
+                                          ~static_cast<uintptr_t>(127));
   __syncthreads();  // (a multi-problem block's previous work item is done with `st`)
   if (threadIdx.x == 0) {
     pass_b_advance<P>(a, bid, nblk, st.ahead, true);
@@ -993,7 +1001,7 @@ __device__ __forceinline__ bool pass_b_run(const PassArgs& a, int bid, int nblk,
           tmem_store_done();
           jcur = pkey * 16 + j;
         }
-      } else {
+      } else if (!chirp_global) {
         ensure_chirp_key<P>(chs, a.chirp_zhat, j, pkey * 16 + j, jcur);
       }
     }
@@ -1054,6 +1062,9 @@ __device__ __forceinline__ bool pass_b_run(const PassArgs& a, int bid, int nblk,
                 for (int i = 0; i < 4; ++i) x[k + i] = cmul(x[k + i], ch[i]);
               }
             } else {
+              // (the first P/2 + 1 entries of the table in global memory are the half table)
+              const ChirpAt<P> cat(
+                  chirp_global ? a.chirp_zhat + (long long)peek(pl.j) * P : chs, t);
 #pragma unroll
               for (int c = 0; c < E; ++c) x[c] = cmul(x[c], cat(c));
             }
@@ -1196,7 +1207,7 @@ constexpr int pass_b_minb() {
 
 template <int P, bool HALF>
 __global__ void __launch_bounds__(ColCfg<P>::NT, pass_b_minb<P, HALF>())
-k_pass_b(const __grid_constant__ PassArgs args) {
+k_pass_b(const __grid_constant__ PassArgs args, int chirp_global) {
   extern __shared__ __align__(16) float2 smem[];
   __shared__ double red[32];
   __shared__ uint64_t ybar;
@@ -1208,21 +1219,23 @@ k_pass_b(const __grid_constant__ PassArgs args) {
   // change are kept in registers or make the compiler copy the loops (at 96 to 168 registers 20 to 550
   // bytes of spills, from shared memory none up to 256 and half at 512; 384^2 on 768^2 206 -> 195 us,
   // 258^2 on 512^2, 24 x 3 planes, 116 -> 107 us).  Longer lines lose by it (512^2 on 1024^2 411 ->
-  // 434 us, 2048^2 on 4096^2 2395 -> 2472 us).
+  // 434 us, 2048^2 on 4096^2 2395 -> 2472 us).  The barrier stays for them as well: without it the
+  // compiler schedules the code behind it differently, 1 to 4 % slower from P = 1024.
   constexpr bool ARGS_SHARED = P <= 768;
   __shared__ PassArgs sargs;
   const PassArgs& a = ARGS_SHARED ? sargs : args;
   if (ARGS_SHARED) {
     for (int i = threadIdx.x; i < (int)(sizeof(PassArgs) / sizeof(int)); i += blockDim.x)
       reinterpret_cast<int*>(&sargs)[i] = reinterpret_cast<const int*>(&args)[i];
-    __syncthreads();
   }
+  __syncthreads();
   Line<P>::load_table(smem, a.twiddles);
   if (threadIdx.x == 0) mbar_init(&ybar);
   __syncthreads();
   uint32_t yphase = 0;
   int jcur = -1;
-  pass_b_run<P, HALF>(a, blockIdx.x, gridDim.x, smem, tbase, red, &ybar, state, yphase, 0, jcur);
+  pass_b_run<P, HALF>(a, blockIdx.x, gridDim.x, smem, tbase, red, &ybar, state, yphase, 0, jcur,
+                      chirp_global != 0);
   __syncthreads();
   if (threadIdx.x < 32) tmem_free(tbase, M::COLS);
 }
@@ -1234,7 +1247,7 @@ k_pass_b(const __grid_constant__ PassArgs args) {
 template <int P, bool HALF>
 __global__ void __launch_bounds__(ColCfg<P>::NT, pass_b_minb<P, HALF>())
 k_pass_b_multi(const PassArgs* __restrict__ args, const int2* __restrict__ items, int nitems,
-               int nprob) {
+               int nprob, int chirp_global) {
   extern __shared__ __align__(16) float2 smem[];
   __shared__ double red[32];
   __shared__ uint64_t ybar;
@@ -1252,7 +1265,7 @@ k_pass_b_multi(const PassArgs* __restrict__ args, const int2* __restrict__ items
     const int2 item = items[it];
     fetch_args(a, args, item.x, cur);
     if (!pass_b_run<P, HALF>(a, item.y, a.pb_blocks, smem, tbase, red, &ybar, state, yphase, item.x,
-                             jcur)) {
+                             jcur, chirp_global != 0)) {
       if (threadIdx.x == 0)
         for (int p = 0; p < nprob; ++p) atomicOr(args[p].err, 1ull);
       break;
@@ -1446,20 +1459,39 @@ cudaError_t launch_cols_sum(const SumArgs& a, const float2* tw, cudaStream_t s) 
 // registers, shared memory and tensor memory.  0: the stage does not fit.  (Counted here: the
 // runtime's occupancy query answers 1 for every kernel that allocates tensor memory.)
 template <int P, bool HALF>
-int pass_b_per_sm(int rows) {
+int pass_b_fit(int rows, bool chirp_global) {
   using Cc = ColCfg<P>;
-  const size_t sm = pass_b_smem<P, HALF>(rows);
+  const size_t sm = pass_b_smem<P, HALF>(rows, chirp_global);
   if (sm > (size_t)max_dynamic_smem()) return 0;
-  cudaFuncAttributes fa;
-  if (cudaFuncGetAttributes(&fa, k_pass_b<P, HALF>) != cudaSuccess || fa.numRegs < 1) {
-    cudaGetLastError();
-    return 1;
+  // (registers and static shared memory of the kernel, the same on every device: asked for once)
+  static std::atomic<int> regs{0}, fixed{0};
+  if (regs.load(std::memory_order_acquire) < 1) {
+    cudaFuncAttributes fa;
+    if (cudaFuncGetAttributes(&fa, k_pass_b<P, HALF>) != cudaSuccess || fa.numRegs < 1) {
+      cudaGetLastError();
+      return 1;
+    }
+    fixed.store((int)fa.sharedSizeBytes, std::memory_order_relaxed);
+    regs.store(fa.numRegs, std::memory_order_release);
   }
   const int warps = (Cc::NT + 31) / 32;
-  const int by_regs = 65536 / ((fa.numRegs + 7) / 8 * 256 * warps);
-  const int by_smem = (int)((size_t)max_sm_smem() / (sm + fa.sharedSizeBytes + 1024));
+  const int by_regs = 65536 / ((regs.load() + 7) / 8 * 256 * warps);
+  const int by_smem = (int)((size_t)max_sm_smem() / (sm + fixed.load() + 1024));
   const int b = std::min({by_regs, by_smem, PassBMem<P, HALF>::MAXB, 64 / warps, 32});
   return b < 1 ? 1 : b;
+}
+// Whether the general forms read the chirp from global memory: where the Y stage would cost a
+// resident block with the chirp in shared memory.  That is the case from P = 2048 for boxes of more
+// than about P/4 rows, which had no stage before: pass B of 2050^2 on 4096^2, 8 x 4 planes, 3535 ->
+// 2550 us, of 1218^2 on 2048^2, 24 x 3 planes, 2077 -> 1815 us.
+template <int P, bool HALF>
+bool pass_b_chirp_global(int rows) {
+  return PassBMem<P, HALF>::CHIRP_ANY && rows > 0 &&
+         pass_b_fit<P, HALF>(rows, false) < pass_b_fit<P, HALF>(0, false);
+}
+template <int P, bool HALF>
+int pass_b_per_sm(int rows) {
+  return pass_b_fit<P, HALF>(rows, pass_b_chirp_global<P, HALF>(rows));
 }
 template <int P>
 int pass_b_per_sm_form(int half, int rows) {
@@ -1487,7 +1519,9 @@ int pass_b_stage_ok(int half, int rows) {
 template <int P, bool HALF>
 cudaError_t launch_pass_b_form(const PassArgs& a, int nblocks, cudaStream_t s) {
   using Cc = ColCfg<P>;
-  const size_t sm = pass_b_smem<P, HALF>(a.ymap ? a.max_box_rows : 0);
+  const int rows = a.ymap ? a.max_box_rows : 0;
+  const bool chirp_global = pass_b_chirp_global<P, HALF>(rows);
+  const size_t sm = pass_b_smem<P, HALF>(rows, chirp_global);
   // (the largest carveout: the driver's own choice follows the occupancy query above)
   cudaError_t e = cudaFuncSetAttribute(k_pass_b<P, HALF>,
                                        cudaFuncAttributePreferredSharedMemoryCarveout,
@@ -1495,7 +1529,7 @@ cudaError_t launch_pass_b_form(const PassArgs& a, int nblocks, cudaStream_t s) {
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(k_pass_b<P, HALF>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
   if (e != cudaSuccess) return e;
-  k_pass_b<P, HALF><<<nblocks, Cc::NT, sm, s>>>(a);
+  k_pass_b<P, HALF><<<nblocks, Cc::NT, sm, s>>>(a, chirp_global);
   const int ngroups = (a.n + Cc::C - 1) / Cc::C, tail = ngroups - (ngroups / nblocks) * nblocks;
   if (a.adj && a.pb_split && tail > 0) {
     e = cudaGetLastError();
@@ -1543,7 +1577,8 @@ cudaError_t launch_pass_b_multi_form(const PassArgs* args, const int2* items, in
                                      int nprob, int max_rows, int per_sm, cudaStream_t s) {
   using Cc = ColCfg<P>;
   if (nitems <= 0) return cudaSuccess;
-  const size_t sm = pass_b_smem<P, HALF>(max_rows);
+  const bool chirp_global = pass_b_chirp_global<P, HALF>(max_rows);
+  const size_t sm = pass_b_smem<P, HALF>(max_rows, chirp_global);
   auto kern = k_pass_b_multi<P, HALF>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout,
                                        cudaSharedmemCarveoutMaxShared);
@@ -1552,7 +1587,7 @@ cudaError_t launch_pass_b_multi_form(const PassArgs* args, const int2* items, in
   if (e != cudaSuccess) return e;
   const int fit = std::max(pass_b_per_sm<P, HALF>(max_rows), 1);  // (registers as k_pass_b's bound)
   const int nb = std::min((per_sm > 0 ? std::min(per_sm, fit) : fit) * sm_count(), nitems);
-  kern<<<nb, Cc::NT, sm, s>>>(args, items, nitems, nprob);
+  kern<<<nb, Cc::NT, sm, s>>>(args, items, nitems, nprob, chirp_global);
   return cudaGetLastError();
 }
 
