@@ -1,11 +1,13 @@
 """The passes' general forms (a side other than P/2, probe shifts) against the oracle: pass B with the
-chirp in shared memory and, for tall boxes at P = 2048 and 4096, in global memory.  Tolerances as in
+chirp in shared memory and, for tall boxes at P = 2048 and 4096, in global memory; and the batch of
+problems of one line length whose general forms share their launches.  Tolerances as in
 test_gpu_parity.py: loss 1e-5, gradients 1e-4 (relative L2)."""
 
 import numpy as np
 import pytest
 
 import test_gpu_parity as plain
+import test_gpu_probe_shift as shifted
 from oracle import holo as oh
 
 pytestmark = pytest.mark.gpu
@@ -42,3 +44,41 @@ def test_general_form_with_and_without_the_stage(n, P, K, J, stage):
     assert loss_f == loss
     check(loss, gp, gq, oh.gradients(pr["psi"], pr["q"], pr["t"], pr["sqrt_d"], pr["sqrt_dref"],
                                      pr["geo"]))
+
+
+def test_batch_of_shifted_and_unshifted_problems():
+    """Problems of one line length, with and without probe shifts, staged and not, in one batch:
+    every problem's results are those of its own calls bit for bit and match the oracle.  (With
+    probe shifts the reference field is part of the full-grid rows; added in pass B once more it
+    made the results of such a batch wrong.)"""
+    from paper_2407_20304_gb300.batch import HoloBatch, Instance
+    insts, refs = [], []
+    for i, (n, P, K, J, ps) in enumerate([(64, 128, 3, 2, True), (64, 128, 2, 4, False),
+                                          (50, 128, 3, 3, False), (96, 192, 2, 2, True),
+                                          (72, 192, 2, 2, False), (128, 128, 2, 1, True),
+                                          (514, 1024, 1, 2, False), (512, 1024, 1, 2, True),
+                                          (608, 2048, 1, 1, False), (1026, 2048, 1, 2, False)]):
+        mod = shifted if ps else plain
+        pr = mod.make_problem(n, P, K, J=J, seed=100 + i, point="object")
+        h = mod.make_holo(pr, chunk=min(2, K))
+        kw = {"probe_shifts": pr["s"]} if ps else {}
+        refs.append(oh.gradients(pr["psi"], pr["q"], pr["t"], pr["sqrt_d"], pr["sqrt_dref"],
+                                 pr["geo"], **kw))
+        insts.append(Instance(h, plain.dev(pr["psi"], torch.complex64),
+                              plain.dev(pr["q"], torch.complex64)))
+    b = HoloBatch(insts)
+    b.prepare_persistent()
+    b.run_loop()
+    torch.cuda.synchronize()
+    own = [(it.h.read_loss(), it.grad_psi.clone(), it.grad_q.clone()) for it in b.inst]
+    for it in b.inst:
+        it.grad_psi.fill_(float("nan"))
+        it.grad_q.fill_(float("nan"))
+    b.capture_persistent()
+    b.replay_persistent()
+    torch.cuda.synchronize()
+    for it, (loss, gp, gq), ref in zip(b.inst, own, refs):
+        assert it.h.read_loss() == loss
+        assert torch.equal(it.grad_psi, gp) and torch.equal(it.grad_q, gq)
+        check(loss, gp, gq, ref)
+    b.close()
