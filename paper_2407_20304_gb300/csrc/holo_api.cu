@@ -351,7 +351,9 @@ struct PassTimer {
 // much.)  The chirp tables carry the inverse of the two factors of a propagation.
 double line_scale(int P) {
   if (P % 3 == 0 && P > 768) return 1.0;
-  const int E = P % 3 == 0 ? 16 : (P >= 512 ? 32 : 16), T = P % 3 == 0 ? P / 48 : P / E;
+  // E: the values per thread, without the factor 3
+  const int E = P % 3 == 0 ? (P > 192 ? 16 : 8) : (P >= 512 ? 32 : 16);
+  const int T = P / (P % 3 == 0 ? 3 * E : E);
   const int T2 = std::min(T, E);
   const double pi = 3.14159265358979323846;
   auto dev = [&](int j, int n) {  // |W_n^j| - 1 after rounding
@@ -395,7 +397,8 @@ std::vector<float2> twiddle_table(int P) {
   const double pi = 3.14159265358979323846;
   auto push = [&](double a) { tw.push_back(make_float2((float)std::cos(a), (float)std::sin(a))); };
   if (P % 3 || P <= 768) {
-    const int E = P % 3 == 0 ? 48 : (P >= 512 ? 32 : 16), T = P / E, T2 = std::min(T, E);
+    const int E = P % 3 == 0 ? (P > 192 ? 48 : 24) : (P >= 512 ? 32 : 16);
+    const int T = P / E, T2 = std::min(T, E);
     for (int m = 1; m < T2; m *= 2)
       for (int k = 0; k < E; ++k) push(-2.0 * pi * (double)k * m / (E * T2));
     if (T > E)

@@ -81,7 +81,7 @@ struct RowCfg {
   static constexpr int LS =
       L::SMEM + (L::R3 ? 0 : (T >= 16 ? 0 : (T == 8 ? 8 : (T == 4 ? 4 : 2))));
   static constexpr size_t SMEM_BYTES = (size_t)(SmemHead<P>::WORDS + G * LS) * sizeof(float2);
-  static constexpr int MINB = L::R3 ? 2 : (P >= 2048 ? 2 : (L::M3 ? 3 : (P >= 512 ? 4 : 6)));
+  static constexpr int MINB = L::R3 ? 2 : (P >= 2048 ? 2 : (L::E == 48 ? 3 : (L::M3 || P >= 512 ? 4 : 6)));
 };
 
 // Column passes: C adjacent columns interleaved in the lanes, so that one access covers the C
@@ -651,7 +651,7 @@ __device__ __forceinline__ void pass_c_step(const PassArgs& a, int s, int next, 
   // transposed taps of this plane (same FP64-built weights as the forward taps); the buffer
   // holds conj(z).
   const float4* xa = reinterpret_cast<const float4*>(a.xadj + (long long)gp * n);
-  constexpr int EH = HALF ? E / 2 : E, CT = EH < 16 ? EH : (E == 48 ? 12 : 16);
+  constexpr int EH = HALF ? E / 2 : E, CT = EH < 16 ? EH : (E % 16 || E == 48 ? 12 : 16);
 #pragma unroll
   for (int c0 = 0; c0 < EH; c0 += CT) {
     float4 tp[CT];  // (the position's bits, both weights; loaded ahead of the barrier)
@@ -1194,7 +1194,7 @@ __device__ __forceinline__ bool pass_b_run(const PassArgs& a, int bid, int nblk,
 
 // Resident blocks that the registers must allow, hence the registers a thread may take: 128 at two
 // blocks of 256 threads (P = 2048, 4096) or four of 128 (512, 1024), 96 at five (up to 256), 168 at
-// three (3 * 2^k, n = P/2 form) and 255 at two (its general form, whose b and S leave room for two
+// three (3 * 2^k) and 255 at two (the general form at 384 and 768, whose b and S leave room for two
 // blocks in tensor memory: with the bound at three it kept to 168 registers and spilled 550 bytes, but
 // two blocks ran all the same; 768^2 on 768^2, 24 x 3 planes: 1330 -> 710 us).  P = 1536 and 3072: one
 // block of 384 threads.

@@ -33,7 +33,11 @@
 // the conjugate of the forward transform of the conjugate, and forward and inverse run as two
 // turns of a loop over one copy of the code (17 KB).
 //
-// P = 3 * 2^k, 48 .. 768: the same two stages with E = 48 (stage 1 is 3 x 16 without twiddles).
+// P = 3 * 2^k, 48 .. 768: the same two stages with E = 24 up to 192 and E = 48 above (stage 1 is 3 x 8
+// or 3 x 16 without twiddles).  At P <= 192 all the work is on the chip in one wave, and 48 values in
+// half the threads only made it longer (96^2 on 96^2, 2 x 4 planes: pass A 19.6 -> 10 us, B 26.3 ->
+// 12.5 us; 98^2 on 192^2, 24 x 3 planes, A and C 33.2 -> 20.0 us).  384 and 768 need rows of 16 values,
+// which 24 values do not give a whole number of.
 // 1536 and 3072 would need 48 rows over 32 or 64 threads: the radix-3 step and the 16-value engine
 // of holo_fft.cuh (E = 16, T = P/16).
 //
@@ -176,29 +180,32 @@ __device__ __forceinline__ void dft_const_zin(float2* v) {
   });
 }
 
-// DFT of length 48 as 3 x 16 without twiddles (Good-Thomas: element (16 a + 3 b) mod 48, output k
-// with k mod 3 and k mod 16 the two indices); X[k] is left in v[dft48_at(k)].
-__host__ __device__ constexpr int dft48_at(int k) {
-  return (16 * (k % 3) + 3 * bit_reverse(k % 16, 4)) % 48;
+// DFT of length 3 B (B = 8 or 16) as 3 x B without twiddles (Good-Thomas: element (B a + 3 b) mod
+// 3 B, output k with k mod 3 and k mod B the two indices); X[k] is left in v[dft3_at<B>(k)].
+template <int B>
+__host__ __device__ constexpr int dft3_at(int k) {
+  return (B * (k % 3) + 3 * bit_reverse(k % B, ilog2c(B))) % (3 * B);
 }
-__device__ __forceinline__ void dft48(float2* v) {
+template <int B>
+__device__ __forceinline__ void dft3(float2* v) {
   static_for<3>([&](auto ac) HOLO_INLINE {
     constexpr int a = decltype(ac)::value;
-    float2 y[16];
-    static_for<16>([&](auto bc) HOLO_INLINE {
+    float2 y[B];
+    static_for<B>([&](auto bc) HOLO_INLINE {
       constexpr int b = decltype(bc)::value;
-      y[b] = v[(16 * a + 3 * b) % 48];
+      y[b] = v[(B * a + 3 * b) % (3 * B)];
     });
-    dft_const_levels<16, 1, 16>(y);
-    static_for<16>([&](auto bc) HOLO_INLINE {
+    dft_const_levels<B, 1, B>(y);
+    static_for<B>([&](auto bc) HOLO_INLINE {
       constexpr int b = decltype(bc)::value;
-      v[(16 * a + 3 * b) % 48] = y[b];
+      v[(B * a + 3 * b) % (3 * B)] = y[b];
     });
   });
   const float h = 0.86602540378443865f;  // sqrt(3)/2
-  static_for<16>([&](auto bc) HOLO_INLINE {
+  static_for<B>([&](auto bc) HOLO_INLINE {
     constexpr int b = decltype(bc)::value;
-    float2 &x0 = v[(3 * b) % 48], &x1 = v[(16 + 3 * b) % 48], &x2 = v[(32 + 3 * b) % 48];
+    float2 &x0 = v[(3 * b) % (3 * B)], &x1 = v[(B + 3 * b) % (3 * B)],
+           &x2 = v[(2 * B + 3 * b) % (3 * B)];
     const float2 su = cadd(x1, x2), df = csub(x1, x2);
     const float2 m = make_float2(fmaf(-0.5f, su.x, x0.x), fmaf(-0.5f, su.y, x0.y));
     x0 = cadd(x0, su);
@@ -241,12 +248,12 @@ template <int P_>
 struct Line<P_, false> {
   static constexpr int P = P_;
   static constexpr bool R3 = false;
-  static constexpr bool M3 = P % 3 == 0;            // P = 3 * 2^k: E = 48
+  static constexpr bool M3 = P % 3 == 0;            // P = 3 * 2^k: E = 48, up to 192 24
   static_assert(is_pow2c(M3 ? P / 3 : P) && P >= 16 && P <= 4096, "line length");
-  static constexpr int E = M3 ? 48 : (P >= 512 ? 32 : 16);
+  static constexpr int E = M3 ? (P > 192 ? 48 : 24) : (P >= 512 ? 32 : 16);
   // where stage 1 leaves output k
   __host__ __device__ static constexpr int at(int k) {
-    return M3 ? dft48_at(k) : bit_reverse(k, ilog2c(E));
+    return M3 ? dft3_at<E / 3>(k) : bit_reverse(k, ilog2c(E));
   }
   static constexpr int T = P / E;
   static constexpr int R = T > E ? T / E : 1;      // radix of the third stage
@@ -281,7 +288,7 @@ struct Line<P_, false> {
         for (int c = 0; c < E; ++c)
           if (c < E / 4 || c >= 3 * E / 4) v[c] = make_float2(0.f, 0.f);
       }
-      dft48(v);
+      dft3<E / 3>(v);
     } else {
       if (ZIN && zin)
         dft_const_zin<E>(v);
