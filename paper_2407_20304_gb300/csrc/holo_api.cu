@@ -344,23 +344,47 @@ struct PassTimer {
 };
 
 
-// The mean factor 1 + d by which a transform of holo_line.cuh scales its values because its
-// constant twiddles are rounded to FP32: |W| of a rounded constant W is 1 + d_W, and a butterfly
-// a +- W b of equally strong a and b scales both by 1 + d_W / 2.  (-7.3e-8 at P = 4096; the four
-// transforms of a plane left u 3e-7 too small, most of its error, and moved the loss twice as
-// much.)  The chirp tables carry the inverse of the two factors of a propagation.
+// The mean factor 1 + d by which a transform scales its values because its twiddles are rounded to
+// FP32: |W| of a rounded W is 1 + d_W.  A butterfly a +- W b of equally strong a and b (holo_line.cuh)
+// scales both by 1 + d_W / 2; a stage that multiplies all its values by twiddles and takes a DFT of
+// them (holo_fft.cuh) by their mean 1 + d_W, and there the 15 powers of one root multiply its error.
+// (-7.3e-8 at P = 4096, -1.06e-7 at 1536: the four transforms of a plane left u 3e-7 and 4e-7 too
+// small, most of its error, and moved the loss twice as much.)  The chirp tables carry the inverse of
+// the two factors of a propagation.
 double line_scale(int P) {
-  if (P % 3 == 0 && P > 768) return 1.0;
+  const double pi = 3.14159265358979323846;
+  auto root = [&](int j, int n) {
+    return make_float2((float)std::cos(2.0 * pi * j / n), (float)-std::sin(2.0 * pi * j / n));
+  };
+  auto off = [](float2 w) { return std::sqrt((double)w.x * w.x + (double)w.y * w.y) - 1.0; };
+  auto dev = [&](int j, int n) { return 4 * j % n == 0 ? 0.0 : off(root(j, n)); };
+  double d = 0.0;
+  if (P % 3 == 0) {  // radix-3 step: of two of its three outputs two thirds carry sqrt(3)/2
+    const double h = (float)std::sqrt(0.75);
+    d += 4.0 / 9.0 * (std::sqrt(0.25 + h * h) - 1.0);
+  }
+  if (P % 3 == 0 && P > 768) {
+    const int PB = P / 3;
+    for (int i = 0; i < 16; ++i) d += 2.0 / 16.0 * dev(i / 4 * (i % 4), 16);  // two radix-16 stages
+    auto mul = [](float2 a, float2 b) {  // as cmul on the device
+      return make_float2(std::fma(a.x, b.x, -a.y * b.y), std::fma(a.x, b.y, a.y * b.x));
+    };
+    for (int L = 1; L <= 16; L *= 16) {  // their twiddles, as pow_apply forms them
+      const int M = PB / (16 * L);
+      for (int mu = 0; mu < M; ++mu) {
+        float2 w[16];
+        w[1] = root(mu * L, PB);
+        for (int k = 2; k < 16; ++k) w[k] = mul(w[k > 8 ? 8 : k > 4 ? 4 : k > 2 ? 2 : 1],
+                                                w[k > 8 ? k - 8 : k > 4 ? k - 4 : k > 2 ? k - 2 : 1]);
+        for (int k = 1; k < 16; ++k) d += off(w[k]) / (16.0 * M);
+      }
+    }
+    return 1.0 + d;
+  }
   // E: the values per thread, without the factor 3
   const int E = P % 3 == 0 ? (P > 192 ? 16 : 8) : (P >= 512 ? 32 : 16);
   const int T = P / (P % 3 == 0 ? 3 * E : E);
   const int T2 = std::min(T, E);
-  const double pi = 3.14159265358979323846;
-  auto dev = [&](int j, int n) {  // |W_n^j| - 1 after rounding
-    const double x = (float)std::cos(2.0 * pi * j / n), y = (float)std::sin(2.0 * pi * j / n);
-    return 4 * j % n == 0 ? 0.0 : std::sqrt(x * x + y * y) - 1.0;
-  };
-  double d = 0.0;
   for (int m = 1; m < E; m *= 2)  // stage 1: the level's m twiddles
     for (int j = 0; j < m; ++j) d += 0.5 * dev(j, 2 * m) / m;
   for (int m = 2; m < T2; m *= 2)  // stage 2: m/2 constants (and -i times them) on table entries

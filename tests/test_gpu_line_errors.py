@@ -16,7 +16,7 @@ pytestmark = pytest.mark.gpu
 torch = pytest.importorskip("torch")
 
 
-@pytest.mark.parametrize("P", [1 << k for k in range(4, 13)] + [3 << k for k in range(4, 9)])
+@pytest.mark.parametrize("P", [1 << k for k in range(4, 13)] + [3 << k for k in range(4, 11)])
 def test_coherent_and_random_error(P):
     if not torch.cuda.is_available():
         pytest.skip("no GPU")
