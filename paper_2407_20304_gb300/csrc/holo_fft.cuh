@@ -1,5 +1,5 @@
-// Register + shared-memory FFT engine of the line lengths P = 3 PB (PB = 2^k, 16 .. 1024), and
-// the complex helpers shared with holo_line.cuh.
+// Register + shared-memory FFT engine of the line lengths P = 1536 and 3072 (P = 3 PB, PB = 512 and
+// 1024), and the complex helpers shared with holo_line.cuh.
 //
 // The Fresnel operator D_z (Appendix A, Eq. defPz/defGz) is a circular convolution on
 // the P x P grid; with a separable chirp exp(-i pi lambda z (fx^2 + fy^2)) it factors into
@@ -8,9 +8,8 @@
 //
 // Sub-line of length PB: TB = PB/16 threads, 16 complex values per thread: thread t, register c
 // holds element t + TB c ("strided natural" layout).  The forward transform is a mixed-radix
-// decimation in frequency with radices 16, 16, ..., 16, r (r in {2, 4, 8} when log2 PB is not a
-// multiple of 4); every stage is a DFT over one digit in registers followed by a twiddle and a
-// shared-memory exchange.  The thread/register assignment of each stage is chosen so that the
+// decimation in frequency with radices 16, 16, R (R = 2 or 4); every stage is a DFT over one digit
+// in registers followed by a twiddle and a shared-memory exchange.  The thread/register assignment of each stage is chosen so that the
 // forward output is again in strided natural order, so a pointwise multiplier in frequency needs
 // no reordering and the inverse transform (the adjoint stages in reverse order) consumes that
 // layout directly and returns the same layout.
@@ -75,10 +74,6 @@ __device__ __forceinline__ float2 cmul(float2 a, float2 b) {
 __device__ __forceinline__ float2 cmulc(float2 a, float2 b) {
   return make_float2(fmaf(a.x, b.x, a.y * b.y), fmaf(a.y, b.x, -a.x * b.y));
 }
-// conj(a) * b
-__device__ __forceinline__ float2 cconjmul(float2 a, float2 b) {
-  return make_float2(fmaf(a.x, b.x, a.y * b.y), fmaf(a.x, b.y, -a.y * b.x));
-}
 __device__ __forceinline__ float2 cscale(float2 a, float s) { return make_float2(a.x * s, a.y * s); }
 __device__ __forceinline__ float2 cconj(float2 a) { return make_float2(a.x, -a.y); }
 // multiply by -i (forward) or +i (inverse)
@@ -93,45 +88,46 @@ __host__ __device__ constexpr int ilog2c(int x) { return x <= 1 ? 0 : 1 + ilog2c
 __host__ __device__ constexpr int ipow16(int s) { return s == 0 ? 1 : 16 * ipow16(s - 1); }
 
 __device__ __forceinline__ int spad(int a) { return a + (a >> 4); }
-__host__ __device__ constexpr int spad_c(int a) { return a + (a >> 4); }
 
 __host__ __device__ constexpr bool is_pow2c(int x) { return x > 0 && (x & (x - 1)) == 0; }
+
+// A sub-line: two radix-16 stages, then one of radix R.  Stage s: prefix length 16^s, remaining length
+// M(s) = PB / 16^(s+1).
+template <int PB>
+struct SubLine {
+  static_assert(PB == 512 || PB == 1024, "sub-line length");
+  static constexpr int T = PB / 16;                // threads
+  static constexpr int N16 = 2;                    // radix-16 stages
+  static constexpr int R = PB / 256;               // radix of the last stage
+  static constexpr int SMEM = PB + PB / 16;        // padded exchange buffer, float2 entries
+  __host__ __device__ static constexpr int M(int s) { return PB / ipow16(s + 1); }
+  // twiddle table in global memory: 15 M(s) entries a stage; in shared memory the roots
+  // W_PB^{mu 16^s} (k = 1) of every stage only
+  __host__ __device__ static constexpr int tw_off(int s) {
+    return s == 0 ? 0 : tw_off(s - 1) + 15 * M(s - 1);
+  }
+  __host__ __device__ static constexpr int roots_off(int s) {
+    return s == 0 ? 0 : roots_off(s - 1) + M(s - 1);
+  }
+};
 
 template <int P_>
 struct Fft {
   static constexpr int P = P_;
-  static constexpr bool R3 = P % 3 == 0;           // one radix-3 step, then three sub-lines
-  static constexpr int PB = R3 ? P / 3 : P;        // power-of-two (sub-)line length
-  static_assert(is_pow2c(PB) && PB >= 16, "line length must be 2^k or 3 * 2^k with 2^k >= 16");
-  static constexpr int LOG2 = ilog2c(PB);
+  static constexpr int PB = P / 3;                 // sub-line length
+  using S = SubLine<PB>;
   static constexpr int T = P / 16;                 // threads per line
-  static constexpr int TB = PB / 16;               // threads per power-of-two sub-line
-  static constexpr int N16 = LOG2 / 4;             // radix-16 stages
-  static constexpr int RB = LOG2 % 4;              // bits of the final small stage (0: none)
-  static constexpr int NST = N16 + (RB ? 1 : 0);   // number of stages
-  static constexpr int RLAST = RB ? (1 << RB) : 16;
-  static constexpr int SMEM = P + P / 16;          // padded exchange buffer, float2 entries
-  // radix-16 stage s: prefix length L = 16^s, remaining length M = PB / 16^(s+1)
-  __host__ __device__ static constexpr int L(int s) { return ipow16(s); }
-  __host__ __device__ static constexpr int M(int s) { return PB / ipow16(s + 1); }
-  __host__ __device__ static constexpr int tw_off(int s) {
-    return s == 0 ? 0 : tw_off(s - 1) + (M(s - 1) > 1 ? 15 * M(s - 1) : 0);
-  }
-  static constexpr int TW_BASE = tw_off(N16);      // radix-16 twiddle entries (float2)
-  // compact table of the roots W_PB^{mu L(s)} (k = 1 entries) of every twiddled stage
-  __host__ __device__ static constexpr int roots_off(int s) {
-    return s == 0 ? 0 : roots_off(s - 1) + (M(s - 1) > 1 ? M(s - 1) : 0);
-  }
-  static constexpr int ROOTS_BASE = roots_off(N16);
+  static constexpr int TB = S::T;                  // threads per sub-line
+  static constexpr int SMEM = 3 * S::SMEM;
   // radix-3 step: W_P^n and W_P^{2n}, n < PB, appended to both tables
-  static constexpr int TW = TW_BASE + (R3 ? 2 * PB : 0);
-  static constexpr int ROOTS = ROOTS_BASE + (R3 ? 2 * PB : 0);
+  static constexpr int TW_BASE = S::tw_off(S::N16), TW = TW_BASE + 2 * PB;
+  static constexpr int ROOTS_BASE = S::roots_off(S::N16), ROOTS = ROOTS_BASE + 2 * PB;
   // line element held in register c of thread t, and the frequency it holds after fft_fwd
   __host__ __device__ static constexpr int pos(int t, int c) {
-    return R3 ? t % TB + TB * c + PB * (t / TB) : t + T * c;
+    return t % TB + TB * c + PB * (t / TB);
   }
   __host__ __device__ static constexpr int fpos(int t, int c) {
-    return R3 ? 3 * (t % TB + TB * c) + t / TB : t + T * c;
+    return 3 * (t % TB + TB * c) + t / TB;
   }
 };
 
@@ -155,27 +151,6 @@ __device__ __forceinline__ void dft4(float2& x0, float2& x1, float2& x2, float2&
   const float2 p = make_float2(d02.x + e.y, d02.y - e.x), m = make_float2(d02.x - e.y, d02.y + e.x);
   x1 = INV ? m : p;
   x3 = INV ? p : m;
-}
-
-template <bool INV>
-__device__ __forceinline__ void dft8(float2* v) {
-  // radix-2 decimation in time over two DFT-4s
-  float2 e0 = v[0], e1 = v[2], e2 = v[4], e3 = v[6];
-  float2 o0 = v[1], o1 = v[3], o2 = v[5], o3 = v[7];
-  dft4<INV>(e0, e1, e2, e3);
-  dft4<INV>(o0, o1, o2, o3);
-  const float h = 0.70710678118654752f;
-  // W8^1 = (1 - i)/sqrt2 forward, (1 + i)/sqrt2 inverse
-  float2 t1 = INV ? make_float2((o1.x - o1.y) * h, (o1.x + o1.y) * h)
-                  : make_float2((o1.x + o1.y) * h, (o1.y - o1.x) * h);
-  float2 t2 = mul_mi<INV>(o2);
-  // W8^3 = (-1 - i)/sqrt2 forward, (-1 + i)/sqrt2 inverse
-  float2 t3 = INV ? make_float2((-o3.x - o3.y) * h, (o3.x - o3.y) * h)
-                  : make_float2((o3.y - o3.x) * h, (-o3.x - o3.y) * h);
-  v[0] = cadd(e0, o0); v[4] = csub(e0, o0);
-  v[1] = cadd(e1, t1); v[5] = csub(e1, t1);
-  v[2] = cadd(e2, t2); v[6] = csub(e2, t2);
-  v[3] = cadd(e3, t3); v[7] = csub(e3, t3);
 }
 
 // W16^m as (cos, -sin) of 2 pi m / 16 (conjugated for the inverse)
@@ -222,22 +197,16 @@ __device__ __forceinline__ void dft16(float2* v) {
 
 template <int R, bool INV>
 __device__ __forceinline__ void dft_small(float2* u) {
-  if constexpr (R == 2) {
+  if constexpr (R == 2)
     dft2<INV>(u[0], u[1]);
-  } else if constexpr (R == 4) {
+  else
     dft4<INV>(u[0], u[1], u[2], u[3]);
-  } else if constexpr (R == 8) {
-    dft8<INV>(u);
-  } else {
-    dft16<INV>(u);
-  }
 }
 
 // --------------------------------------------------------------------- twiddle tables
 
 // Host-side layout of the twiddle table of one line length P = 3 PB: for each radix-16
-// stage s with M(s) > 1, entries [(k-1) * M(s) + mu] = exp(-2 pi i mu k L(s) / PB),
-// k = 1..15, mu = 0..M(s)-1; then [n] = exp(-2 pi i n / P) and
+// stage s, entries [(k-1) * M(s) + mu] = exp(-2 pi i mu k 16^s / PB), k = 1..15, mu = 0..M(s)-1; then [n] = exp(-2 pi i n / P) and
 // [PB + n] = exp(-2 pi i 2n / P), n < PB.  Filled in FP64 on the host.
 
 // v[k] times the k-th power of r (its conjugate for INV), k = 1 .. 15: the powers by a product
@@ -259,33 +228,31 @@ __device__ __forceinline__ void pow_apply(float2 (&v)[16], float2 r) {
   for (int k = 1; k < 16; ++k) v[k] = INV ? cmulc(v[k], w[k]) : cmul(v[k], w[k]);
 }
 
-// TwRoots: the powers from the compact root table (Fft<P>::ROOTS entries: k = 1 of every
-// twiddled stage), which is small enough to keep in shared memory next to the chirp.
+// The compact root table (Fft<P>::ROOTS entries: k = 1 of every stage, and the radix-3 step's
+// twiddles), small enough to keep in shared memory next to the chirp.
 struct TwRoots {
   const float2* roots;
   template <int P>
   __device__ __forceinline__ float2 r3(int idx) const {
     return roots[Fft<P>::ROOTS_BASE + idx];
   }
-  template <int P, int S, bool INV>
+  template <int PB, int S, bool INV>
   __device__ __forceinline__ void apply(float2 (&v)[16], int mu) const {
-    pow_apply<INV>(v, roots[Fft<P>::roots_off(S) + mu]);
+    pow_apply<INV>(v, roots[SubLine<PB>::roots_off(S) + mu]);
   }
 };
 
-// Copy the roots of every twiddled stage from the full table (block-wide).
+// Copy the roots of every stage from the full table (block-wide).
 template <int P>
 __device__ __forceinline__ void load_roots(float2* sm_roots, const float2* __restrict__ g_tw) {
   using F = Fft<P>;
+  using B = typename F::S;
 #pragma unroll
-  for (int st = 0; st < F::N16; ++st) {
-    if (F::M(st) > 1)
-      for (int mu = threadIdx.x; mu < F::M(st); mu += blockDim.x)
-        sm_roots[F::roots_off(st) + mu] = g_tw[F::tw_off(st) + mu];
-  }
-  if constexpr (F::R3)
-    for (int i = threadIdx.x; i < 2 * F::PB; i += blockDim.x)
-      sm_roots[F::ROOTS_BASE + i] = g_tw[F::TW_BASE + i];
+  for (int st = 0; st < B::N16; ++st)
+    for (int mu = threadIdx.x; mu < B::M(st); mu += blockDim.x)
+      sm_roots[B::roots_off(st) + mu] = g_tw[B::tw_off(st) + mu];
+  for (int i = threadIdx.x; i < 2 * F::PB; i += blockDim.x)
+    sm_roots[F::ROOTS_BASE + i] = g_tw[F::TW_BASE + i];
 }
 
 // --------------------------------------------------------------------- stages
@@ -294,30 +261,28 @@ __device__ __forceinline__ void load_roots(float2* sm_roots, const float2* __res
 struct SyncBlock {
   __device__ __forceinline__ void operator()() const { __syncthreads(); }
 };
-#define HOLO_SYNC() sync()
 
-template <int P, int S, class Sync = SyncBlock, class TW = TwRoots>
-__device__ __forceinline__ void fwd_from(float2 (&v)[16], float2* __restrict__ sm, TW tw, int t,
-                                         Sync sync = Sync()) {
-  using F = Fft<P>;
+// The sub-line's forward transform from stage S on; thread t, register c hold element t + T c.
+template <int PB, int S, class Sync>
+__device__ __forceinline__ void fwd_from(float2 (&v)[16], float2* __restrict__ sm, TwRoots tw, int t,
+                                         Sync sync) {
+  using F = SubLine<PB>;
   if constexpr (S < F::N16) {
     constexpr int M = F::M(S);
     if constexpr (S > 0) {
       const int mu = t % M, ka = t / M;
 #pragma unroll
       for (int c = 0; c < 16; ++c) v[c] = sm[spad(c * M + mu + 16 * M * ka)];
-      HOLO_SYNC();
+      sync();
     }
     dft16<false>(v);
-    if constexpr (M > 1) tw.template apply<P, S, false>(v, t % M);
-    if constexpr (S < F::NST - 1) {
+    tw.template apply<PB, S, false>(v, t % M);
 #pragma unroll
-      for (int k = 0; k < 16; ++k) sm[spad(t + F::T * k)] = v[k];
-      HOLO_SYNC();
-    }
-    fwd_from<P, S + 1, Sync, TW>(v, sm, tw, t, sync);
-  } else if constexpr (F::RB > 0 && S == F::N16) {
-    constexpr int R = F::RLAST, G = 16 / R;
+    for (int k = 0; k < 16; ++k) sm[spad(t + F::T * k)] = v[k];
+    sync();
+    fwd_from<PB, S + 1>(v, sm, tw, t, sync);
+  } else {
+    constexpr int R = F::R, G = 16 / R;
 #pragma unroll
     for (int g = 0; g < G; ++g) {
       float2 u[R];
@@ -328,56 +293,54 @@ __device__ __forceinline__ void fwd_from(float2 (&v)[16], float2* __restrict__ s
 #pragma unroll
       for (int k = 0; k < R; ++k) v[g + G * k] = u[k];
     }
-    HOLO_SYNC();
+    sync();
   }
 }
 
-template <int P, int S, class Sync = SyncBlock, class TW = TwRoots>
-__device__ __forceinline__ void inv_from(float2 (&v)[16], float2* __restrict__ sm, TW tw, int t,
-                                         Sync sync = Sync()) {
-  using F = Fft<P>;
+// Its adjoint, stages S, S - 1, ..., 0.
+template <int PB, int S, class Sync>
+__device__ __forceinline__ void inv_from(float2 (&v)[16], float2* __restrict__ sm, TwRoots tw, int t,
+                                         Sync sync) {
+  using F = SubLine<PB>;
   if constexpr (S == F::N16) {
-    if constexpr (F::RB > 0) {
-      constexpr int R = F::RLAST, G = 16 / R;
+    constexpr int R = F::R, G = 16 / R;
 #pragma unroll
-      for (int g = 0; g < G; ++g) {
-        float2 u[R];
+    for (int g = 0; g < G; ++g) {
+      float2 u[R];
 #pragma unroll
-        for (int k = 0; k < R; ++k) u[k] = v[g + G * k];
-        dft_small<R, true>(u);
-        const int ka = t + F::T * g;
+      for (int k = 0; k < R; ++k) u[k] = v[g + G * k];
+      dft_small<R, true>(u);
+      const int ka = t + F::T * g;
 #pragma unroll
-        for (int c = 0; c < R; ++c) sm[spad(c + R * ka)] = u[c];
-      }
-      HOLO_SYNC();
-#pragma unroll
-      for (int k = 0; k < 16; ++k) v[k] = sm[spad(t + F::T * k)];
-      HOLO_SYNC();
+      for (int c = 0; c < R; ++c) sm[spad(c + R * ka)] = u[c];
     }
-    inv_from<P, S - 1, Sync, TW>(v, sm, tw, t, sync);
-  } else if constexpr (S >= 0) {
+    sync();
+#pragma unroll
+    for (int k = 0; k < 16; ++k) v[k] = sm[spad(t + F::T * k)];
+    sync();
+    inv_from<PB, S - 1>(v, sm, tw, t, sync);
+  } else {
     constexpr int M = F::M(S);
-    if constexpr (M > 1) tw.template apply<P, S, true>(v, t % M);
+    tw.template apply<PB, S, true>(v, t % M);
     dft16<true>(v);
     if constexpr (S > 0) {
       const int mu = t % M, ka = t / M;
 #pragma unroll
       for (int c = 0; c < 16; ++c) sm[spad(c * M + mu + 16 * M * ka)] = v[c];
-      HOLO_SYNC();
+      sync();
 #pragma unroll
       for (int k = 0; k < 16; ++k) v[k] = sm[spad(t + F::T * k)];
-      HOLO_SYNC();
-      inv_from<P, S - 1, Sync, TW>(v, sm, tw, t, sync);
+      sync();
+      inv_from<PB, S - 1>(v, sm, tw, t, sync);
     }
   }
 }
 
-// Radix-3 steps of P = 3 PB (see the layout notes at the top).  v[c] of thread (q, i) is
-// element n + PB q (n = i + TB c) on entry to r3_split and frequency-side y_q[n] on exit;
-// r3_merge is its adjoint (conjugate twiddles and roots of unity, no 1/3).
-template <int P, bool INV, class Sync, class TW>
-__device__ __forceinline__ void r3_butterfly_third(float2 (&v)[16], float2* __restrict__ sm, TW tw,
-                                                   int t, Sync sync) {
+// The radix-3 butterflies of P = 3 PB: group q takes output q of every butterfly of the elements in
+// sm (n = i + TB c of thread (q, i)); INV: conjugate roots of unity, no 1/3.
+template <int P, bool INV, class Sync>
+__device__ __forceinline__ void r3_butterfly_third(float2 (&v)[16], float2* __restrict__ sm, int t,
+                                                   Sync sync) {
   using F = Fft<P>;
   constexpr int PB = F::PB, TB = F::TB;
   const float h3 = 0.86602540378443865f;  // sqrt(3)/2
@@ -399,32 +362,34 @@ __device__ __forceinline__ void r3_butterfly_third(float2 (&v)[16], float2* __re
     }
     v[c] = y;
   }
-  (void)tw;
   sync();
 }
 
-template <int P, class Sync, class TW>
-__device__ __forceinline__ void r3_fwd(float2 (&v)[16], float2* sm, TW tw, int t, Sync sync) {
+// Forward DFT (e^{-2 pi i}, unnormalised): pos layout in, fpos layout out.
+template <int P, class Sync>
+__device__ __forceinline__ void fft_fwd_with(float2 (&v)[16], float2* sm, TwRoots tw, int t,
+                                             Sync sync) {
   using F = Fft<P>;
   constexpr int PB = F::PB, TB = F::TB;
   const int q = t / TB, i = t % TB;
 #pragma unroll
   for (int c = 0; c < 16; ++c) sm[spad(i + TB * c + PB * q)] = v[c];
   sync();
-  r3_butterfly_third<P, false>(v, sm, tw, t, sync);
+  r3_butterfly_third<P, false>(v, sm, t, sync);
   if (q > 0) {
 #pragma unroll
     for (int c = 0; c < 16; ++c) v[c] = cmul(v[c], tw.template r3<P>((q - 1) * PB + i + TB * c));
   }
-  fwd_from<PB, 0, Sync, TW>(v, sm + q * Fft<PB>::SMEM, tw, i, sync);
+  fwd_from<PB, 0>(v, sm + q * SubLine<PB>::SMEM, tw, i, sync);
 }
-
-template <int P, class Sync, class TW>
-__device__ __forceinline__ void r3_inv(float2 (&v)[16], float2* sm, TW tw, int t, Sync sync) {
+// Inverse DFT without the 1/P factor (the adjoint of fft_fwd_with): fpos in, pos out.
+template <int P, class Sync>
+__device__ __forceinline__ void fft_inv_with(float2 (&v)[16], float2* sm, TwRoots tw, int t,
+                                             Sync sync) {
   using F = Fft<P>;
   constexpr int PB = F::PB, TB = F::TB;
   const int q = t / TB, i = t % TB;
-  inv_from<PB, Fft<PB>::N16, Sync, TW>(v, sm + q * Fft<PB>::SMEM, tw, i, sync);
+  inv_from<PB, SubLine<PB>::N16>(v, sm + q * SubLine<PB>::SMEM, tw, i, sync);
   if (q > 0) {
 #pragma unroll
     for (int c = 0; c < 16; ++c) v[c] = cmulc(v[c], tw.template r3<P>((q - 1) * PB + i + TB * c));
@@ -432,24 +397,7 @@ __device__ __forceinline__ void r3_inv(float2 (&v)[16], float2* sm, TW tw, int t
 #pragma unroll
   for (int c = 0; c < 16; ++c) sm[spad(i + TB * c + PB * q)] = v[c];
   sync();
-  r3_butterfly_third<P, true>(v, sm, tw, t, sync);
+  r3_butterfly_third<P, true>(v, sm, t, sync);
 }
 
-// Forward DFT (e^{-2 pi i}, unnormalised): pos layout in, fpos layout out (both strided
-// natural when P is a power of two).
-template <int P, class Sync, class TW>
-__device__ __forceinline__ void fft_fwd_with(float2 (&v)[16], float2* sm, TW tw, int t, Sync sync) {
-  if constexpr (Fft<P>::R3)
-    r3_fwd<P, Sync, TW>(v, sm, tw, t, sync);
-  else
-    fwd_from<P, 0, Sync, TW>(v, sm, tw, t, sync);
-}
-// Inverse DFT without the 1/P factor (the adjoint of fft_fwd): fpos in, pos out.
-template <int P, class Sync, class TW>
-__device__ __forceinline__ void fft_inv_with(float2 (&v)[16], float2* sm, TW tw, int t, Sync sync) {
-  if constexpr (Fft<P>::R3)
-    r3_inv<P, Sync, TW>(v, sm, tw, t, sync);
-  else
-    inv_from<P, Fft<P>::N16, Sync, TW>(v, sm, tw, t, sync);
-}
 }  // namespace holo
