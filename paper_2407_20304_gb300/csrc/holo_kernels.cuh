@@ -182,14 +182,15 @@ struct ChirpAt {
   const float2* tab;
   int t;
   __device__ __forceinline__ ChirpAt(const float2* tb, int tt) : tab(tb), t(tt) {}
-  __device__ __forceinline__ float2 operator()(int c) const {
+  __host__ __device__ static constexpr int at(int t, int c) {
     if constexpr (L::R3) {
       const int f = L::fpos(t, c);
-      return tab[f <= P / 2 ? f : P - f];
+      return f <= P / 2 ? f : P - f;
     } else {
-      return c < L::E / 2 ? tab[t + L::T * c] : tab[L::T - t + L::T * (L::E - 1 - c)];
+      return c < L::E / 2 ? t + L::T * c : L::T - t + L::T * (L::E - 1 - c);
     }
   }
+  __device__ __forceinline__ float2 operator()(int c) const { return tab[at(t, c)]; }
 };
 
 // Copy the half chirp table of one distance into shared memory (block-wide).

@@ -261,7 +261,8 @@ struct Line<P_, false> {
   static constexpr int T2 = R > 1 ? E : T;         // their length
   // Exchange rows of T values.  Two stages: 16-byte reads of one row per lane, row pitch 4 mod
   // 32 words.  Three stages: 8-byte accesses of one row per lane, odd row pitch.  Either way
-  // every access of a warp is free of bank conflicts.
+  // every access of a warp is free of bank conflicts where a line has 16 threads or more; with
+  // fewer, the writes of a block's many columns take two passes.
   static constexpr int RS = R > 1 ? T + 1 : T + 2;
   static constexpr int SMEM = T > 1 ? E * RS : P;  // float2 entries of a line's buffer (>= P)
   static constexpr int B2 = ilog2c(T2);
