@@ -781,7 +781,7 @@ size_t pass_b_smem(int srows, bool chirp_global) {
   return srows > 0 ? base + 128 + pass_b_stage_bytes<P>(srows) : base;
 }
 
-// Crop rows per run of pass B's loads of b and of the data (a divisor of NS, a multiple of 4).
+// Crop rows per run of pass B's loads (a divisor of NS, a multiple of 4).
 __host__ __device__ constexpr int crop_run(int ns) {
   return ns % 16 == 0 ? 16 : (ns % 12 == 0 ? 12 : 8);
 }
@@ -964,8 +964,10 @@ __device__ __forceinline__ bool pass_b_run(const PassArgs& a, int bid, int nblk,
     if (peek(pl.first)) {
       // (the stores and loads of tensor memory take whole warps)
       const int col = peek(pl.cg) * C + g;
-      // (RUN loads in flight: four at a time the twelve rounds of NS = 48 took 5 us of a small problem)
-      constexpr int RUN = crop_run(NS);
+      // (RUN loads in flight: four at a time the twelve rounds of NS = 48 took 5 us of a small problem.
+      // The n = P/2 forms of 32 and 48 values have 4 or 6 rounds and keep to four: with longer runs
+      // ptxas spills more in the loops below, a batch of sides 256 .. 1024 takes 0.8 % longer)
+      constexpr int RUN = HALF && E >= 32 ? 4 : crop_run(NS);
 #pragma unroll 1
       for (int k = 0; k < NS; k += RUN) {
         float2 x[RUN / 4][4], zero[4];
@@ -1092,7 +1094,7 @@ __device__ __forceinline__ bool pass_b_run(const PassArgs& a, int bid, int nblk,
       float lsum = 0.f;
       // (the loads of RUN crop rows' data are issued together, ahead of their use; all NS at once
       // spill at NS = 32 and 48)
-      constexpr int RUN = crop_run(NS);
+      constexpr int RUN = NS == 24 ? 24 : crop_run(NS);
 #pragma unroll
       for (int k0 = 0; k0 < NS; k0 += RUN) {
         float dat[RUN];
