@@ -410,9 +410,10 @@ std::vector<float2> chirp_table(int P, double lambda, double dx, double z) {
   return c;
 }
 
-// Twiddle table of one line length (FP64).  P = 2^k and 3 * 2^k <= 768, in the layout of holo_line.cuh (E values per
-// thread, T = P/E threads, second stage of T2 = min(T, E)): entries [l E + k1] =
-// exp(-2 pi i k1 2^l / (E T2)), l < log2 T2, k1 < E, then for T > E [t] = exp(-2 pi i t / P).
+// Twiddle table of one line length (FP64).  P = 2^k and 3 * 2^k <= 768, in the layout of
+// holo_line.cuh (E values per thread, T = P/E threads, second stage of T2 = min(T, E)): entries
+// [l E + k1] = exp(-2 pi i k1 2^l / (E T2)), l < log2 T2, k1 < E, then for T > E [t] =
+// exp(-2 pi i t / P).
 // Larger P = 3 PB, in the layout of holo_fft.cuh: radix-16 stage s with M(s) = PB/16^(s+1) > 1
 // contributes entries [(k-1) M + mu] = exp(-2 pi i mu k 16^s / PB), k = 1..15, then the radix-3
 // step adds exp(-2 pi i r n / P) for r = 1, 2 (outer) and n < PB (inner).
@@ -618,12 +619,14 @@ PassArgs pass_args(holo_ctx* c, int k0, int nk, const void* psi) {
 
 // One evaluation is split in three phases so that holo_gradient_host can run the planes of
 // a chunk in parts while copies overlap:
-//   eval_begin:  reference residual r_ref and its loss (only for the chunk with k0 == 0 and
-//                w_ref != 0) into d_red[1], else d_red[1] = 0;
-//   eval_planes: passes A, B (and C, D for gradients) of the angles of `a`; plane loss into
-//                d_red[0] and the call / running totals (k_loss_total); pass B writes or adds
-//                T = ext sum_kj r_kj (+ w_ref r_ref on the first part);
+//   eval_begin:  the reference residual r_ref and its loss partials, which lie behind pass B's in
+//                d_part (only for the chunk with k0 == 0 and w_ref != 0);
+//   eval_planes: passes A, B (and C, D for gradients) of the angles of `a`; pass B writes or adds
+//                T = ext sum_kj r_kj (+ w_ref r_ref on the first part); then eval_loss (one k_loss
+//                launch): the plane loss into d_red[0], on the first part the reference loss into
+//                d_red[1] (0 without one), and the call / running totals;
 //   eval_qgrad:  grad_q of the whole chunk from T and the per-plane conj(w) v.
+
 // Pass B's grid.  Whole column groups go to the blocks in rounds.  When that leaves a partial
 // last round, the (group, plane) items of that round can be spread over all blocks (holo_split.h;
 // pb_split 1: without the Y stage, 2: with it where it fits; automatic when there are fewer than

@@ -11,7 +11,7 @@ namespace holo {
 // One (angle k, distance j) plane: resample parameters and the bounding box of the
 // support of R0(psi - ext) on the P x P grid (rows [by0, by0+bys), cols [bx0, bx0+bxs)).
 // m~ is split into a high part with few significant bits (so m_hi * integer is exact in
-// FP32) and a low part; see axis_tap() in holo_kernels.cuh.
+// FP32) and a low part (the taps of a plane are built on the host, axis_taps in holo_api.cu).
 struct alignas(16) PlaneDesc {
   float mt_hi, mt_lo;   // m~_j = mt_hi + mt_lo
   float ty, tx;         // sample shift t_kj (pixels), (y, x)

@@ -918,10 +918,12 @@ __device__ __noinline__ void pass_b_next(const PassArgs& a, int bid, int nblk, P
 //
 // What bounds it: the transforms themselves (11.7 of 17.4 ms on the 2048^2 chunk of 240 planes, 1.6
 // of 2.8 at 512^2 x 720 planes, alone on the chip), FP32 pipe 48 % and shared memory 51 % busy; the
-// 16-byte pieces of V's stores cost 1.6 ms at P = 4096.  Before (b, S and chirp in shared memory, one
-// block per SM, radix-16 engine): 20.0 and 5.6 ms; 1024^2 x 360 planes 8.9 -> 6.1 ms.  Without the Y
-// stage 22.9 ms.  With the block's work list and descriptors in registers the spills (900 bytes a
-// plane) went to L2: 31.8 ms, so fields are read from shared memory (peek) where they are used.
+// 16-byte pieces of V's stores cost 1.6 ms at P = 4096.  The 128 registers of two 256-thread blocks
+// (four of 128) do not hold a plane's 32 values and all else: 104 to 180 bytes of spills a thread
+// remain in these forms.  Before (b, S and chirp in shared memory, one block per SM, radix-16
+// engine): 20.0 and 5.6 ms; 1024^2 x 360 planes 8.9 -> 6.1 ms.  Without the Y stage 22.9 ms.  With the
+// block's work list and descriptors in registers the spills (900 bytes a plane) went to L2: 31.8 ms,
+// so fields are read from shared memory (peek) where they are used.
 //
 // The block's FP64 loss partial goes to a.loss_part[bid].  The caller has loaded the twiddle
 // table at the head of shared memory and, for a staged problem, initialised the Y-stage barrier.
