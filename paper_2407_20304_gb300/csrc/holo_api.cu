@@ -256,8 +256,8 @@ bool is_pow2(int x) { return x > 0 && (x & (x - 1)) == 0; }
 
 // Pass B's Y stage: a TMA tensor map over ybuf viewed as a row-major [planes * maxbys][2n]
 // float matrix, boxes of 2C floats x stage_box(P) rows.  Used only where the driver provides
-// the encoder, n is even (16-byte row pitch) and the stage leaves pass B's resident blocks
-// per SM unchanged; otherwise pass B loads Y directly.
+// the encoder, n is even (16-byte row pitch) and the stage pays (pass_b_stage_ok); otherwise pass B
+// loads Y directly.
 using EncodeTiledFn = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*,
                                    const cuuint64_t*, const cuuint64_t*, const cuuint32_t*,
                                    const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
@@ -612,7 +612,6 @@ PassArgs pass_args(holo_ctx* c, int k0, int nk, const void* psi) {
   if (c->probe_shift) {
     a.ramp_x = c->d_ramp_x;
     a.ramp_y = c->d_ramp_y;
-    a.ymap = nullptr;
   }
   return a;
 }

@@ -1485,14 +1485,14 @@ int pass_b_fit(int rows, bool chirp_global) {
   const int b = std::min({by_regs, by_smem, PassBMem<P, HALF>::MAXB, 64 / warps, 32});
   return b < 1 ? 1 : b;
 }
-// Whether the general forms read the chirp from global memory: where the Y stage would cost a
-// resident block with the chirp in shared memory.  That is the case from P = 2048 for boxes of more
+// Whether the general forms read the chirp from global memory: where a Y stage has room for more
+// resident blocks without it in shared memory.  That is the case from P = 2048 for boxes of more
 // than about P/4 rows, which had no stage before: pass B of 2050^2 on 4096^2, 8 x 4 planes, 3535 ->
 // 2550 us, of 1218^2 on 2048^2, 24 x 3 planes, 2077 -> 1815 us.
 template <int P, bool HALF>
 bool pass_b_chirp_global(int rows) {
   return PassBMem<P, HALF>::CHIRP_ANY && rows > 0 &&
-         pass_b_fit<P, HALF>(rows, false) < pass_b_fit<P, HALF>(0, false);
+         pass_b_fit<P, HALF>(rows, false) < pass_b_fit<P, HALF>(rows, true);
 }
 template <int P, bool HALF>
 int pass_b_per_sm(int rows) {
@@ -1512,13 +1512,20 @@ int pass_b_blocks(int items, int half, int rows) {
   return (int)(items < b ? items : b);
 }
 
-// The Y stage is used from P = 1024 where the box is at most 256 floats wide, the
-// shared memory fits and pass B keeps its resident blocks per SM.
+// The Y stage is used from P = 1024 where the box is at most 256 floats wide, the shared memory fits
+// and pass B keeps three quarters of its resident blocks per SM, at P = 4096 any.  Loads of Y without
+// it wait where they are issued, and at P = 4096 they are pieces of 16 bytes that get slower the more
+// memory a chunk covers: full-grid boxes of 2048^2 on 4096^2, 60 x 4 planes, 51.2 ms with two blocks
+// without the stage, 35.2 with one and the stage (12 x 4 planes: 7.6, 7.2); 4096^2 on 4096^2, 24 x 3
+// planes, 24.1 and 19.4 (2 x 2 planes: 1.34, 1.57).  512^2 on 1024^2 with full-grid boxes, 40 x 4
+// planes, four blocks 1.36 ms, three and the stage 1.16.  At P = 2048, where one block with the stage
+// would replace two without, 2048^2 on 2048^2, 60 x 3 planes, took 13.0 ms against 10.6.
 template <int P>
 int pass_b_stage_ok(int half, int rows) {
   if (P < 1024 || rows <= 0 || 2 * ColCfg<P>::C > 256) return 0;
   const int b1 = pass_b_per_sm_form<P>(half, rows);
-  return b1 >= 1 && b1 == pass_b_per_sm_form<P>(half, 0) ? 1 : 0;
+  const int b0 = pass_b_per_sm_form<P>(half, 0);
+  return b1 >= 1 && (4 * b1 >= 3 * b0 || P == 4096) ? 1 : 0;
 }
 
 template <int P, bool HALF>

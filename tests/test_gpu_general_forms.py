@@ -82,3 +82,22 @@ def test_batch_of_shifted_and_unshifted_problems():
         assert torch.equal(it.grad_psi, gp) and torch.equal(it.grad_q, gq)
         check(loss, gp, gq, ref)
     b.close()
+
+
+@pytest.mark.parametrize("n,P,K,J", [(512, 1024, 2, 2), (700, 1024, 3, 1), (768, 1536, 1, 2),
+                                     (1024, 2048, 1, 2), (1200, 4096, 2, 1)])
+@pytest.mark.parametrize("stage", [-1, 0])
+def test_probe_shifts_with_and_without_the_stage(n, P, K, J, stage):
+    pr = shifted.make_problem(n, P, K, J=J, seed=19 * n + J, point="object")
+    h = shifted.make_holo(pr)
+    h.set_schedule(0, stage, -1)
+    psi = plain.dev(pr["psi"], torch.complex64)
+    loss_f = h.forward(psi)
+    loss, gp, gq = h.gradient(psi)
+    assert loss_f == loss
+    check(loss, gp, gq, oh.gradients(pr["psi"], pr["q"], pr["t"], pr["sqrt_d"], pr["sqrt_dref"],
+                                     pr["geo"], probe_shifts=pr["s"]))
+    h.set_probe_shifts(None)  # back to the boxes: the stage's tensor map and sizes follow
+    loss_b = h.forward(psi)
+    u = oh.gradients(pr["psi"], pr["q"], pr["t"], pr["sqrt_d"], pr["sqrt_dref"], pr["geo"])[0]
+    assert abs(loss_b - u) / u < plain.LOSS_TOL
